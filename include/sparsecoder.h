@@ -183,9 +183,10 @@ typedef struct {
  * counterpart; this is an interface convenience.
  *
  * Same arguments, semantics and results as sc_layer_forward (the caller still
- * passes every input and output).  The scratch comes from a 6 MiB array
+ * passes every input and output).  The scratch comes from arrays of 22 MiB
  * compiled into the library, which every GPU that loads it holds until the
- * process exits; sizes whose scratch does not fit (from roughly B*L*H = 100k
+ * process exits; sizes whose scratch does not fit the first of them, of 6 MiB
+ * (from roughly B*L*H = 100k
  * (sequence, token, head) rows on; B=2, L=4096, H=12 is 98k and fits) return
  * SC_ERR_UNSUPPORTED with the detail in sc_last_error().  The first call
  * on each device looks up the array's device address (cudaGetSymbolAddress);

@@ -86,7 +86,7 @@ struct WsLayout {
       gathered, gcur, ng,
       ident,
       tail_from,
-      loop_layer, qkv, total;
+      loop_layer, qkv, gprob, gog, total;
 };
 
 bool ws_layout(int B, int L, int H, WsLayout* w) {
@@ -117,6 +117,8 @@ bool ws_layout(int B, int L, int H, WsLayout* w) {
   w->loop_layer = take(sizeof(int32_t));
   // compacted Q, K, V of the current layer (rows of the surviving tokens)
   w->qkv = take(sizeof(uint16_t) * 3 * B * (size_t)L * H * kHeadDim);
+  w->gprob = take(sizeof(float) * B * H * (size_t)L * kMaxGlobal);
+  w->gog = take(sizeof(float) * B * H * T * kMaxGlobal * kHeadDim);
   w->total = off;
   return true;
 }
@@ -316,6 +318,8 @@ void fill_workspace(LayerParams* p, char* ws, const WsLayout& lay, int slot) {
   p->gpart = reinterpret_cast<float*>(ws + lay.gpart);
   p->gstat = reinterpret_cast<float*>(ws + lay.gstat);
   p->og = reinterpret_cast<float*>(ws + lay.og);
+  p->gprob = reinterpret_cast<float*>(ws + lay.gprob);
+  p->gog = reinterpret_cast<float*>(ws + lay.gog);
   p->keep = reinterpret_cast<uint8_t*>(ws + lay.keep);
   p->cnt_tile = reinterpret_cast<uint32_t*>(ws + lay.cnt_tile);
   p->cnt_seq = reinterpret_cast<uint32_t*>(ws + lay.cnt_seq);
@@ -331,12 +335,11 @@ void fill_workspace(LayerParams* p, char* ws, const WsLayout& lay, int slot) {
   p->ng_out = ng + (1 - slot) * p->B;
   p->ident = ident + slot * p->B;
   p->ident_out = ident + (1 - slot) * p->B;
-  // rows kernel layout: pairs of query tiles, or single tiles when a tile's
-  // band reaches more than five key tiles
-  p->wide = (p->w > kPairWindow && p->T > kMaxBandTiles) ? 1 : 0;
-  p->band_slots = p->wide ? kWideBandTiles : kMaxBandTiles;
+  // query tiles whose bands can reach one key tile
+  const bool wide = p->w > kNarrowWindow && p->T > kMaxBandTiles;
+  p->band_slots = wide ? kWideBandTiles : kMaxBandTiles;
   p->sms = device_sms();
-  p->band = (!p->wide && p->sms > 0 &&
+  p->band = (!wide && p->sms > 0 &&
              g_rows_kernel.load(std::memory_order_relaxed) == SC_ROWS_SINGLE_PASS) ? 1 : 0;
 }
 
@@ -1170,19 +1173,25 @@ int sc_workspace_status(void* workspace, size_t ws_bytes, void* stream) {
 namespace {
 
 constexpr size_t kStaticWorkspaceBytes = size_t(6) << 20;  // 6 MiB
+// The global rows' probabilities and output parts: at most 16 MiB for the
+// sizes whose other scratch fits above (40 bytes of it per (sequence, token,
+// head) row against 64 here, and at least half the 4 KB per tile).
+constexpr size_t kStaticGlobalBytes = size_t(16) << 20;
 
 }  // namespace
 
 static __device__ __align__(256) unsigned char g_static_workspace[kStaticWorkspaceBytes];
+static __device__ __align__(256) unsigned char g_static_global[kStaticGlobalBytes];
 
 namespace {
 
-// Device address of g_static_workspace on the current device.  In host code
-// the array's name is only a stand-in, so the address is looked up once per
+// Device addresses of the two arrays on the current device.  In host code an
+// array's name is only a stand-in, so the addresses are looked up once per
 // device (with that device current) and cached.
-int static_workspace(char** out) {
+int static_workspace(char** out, char** global_rows = nullptr) {
   static std::mutex mu;
   static void* addr[256] = {nullptr};
+  static void* gaddr[256] = {nullptr};
   int dev = 0;
   const cudaError_t ge = cudaGetDevice(&dev);
   if (ge != cudaSuccess) return fail_cuda("cudaGetDevice", ge);
@@ -1190,11 +1199,13 @@ int static_workspace(char** out) {
   std::lock_guard<std::mutex> lock(mu);
   if (addr[dev] == nullptr) {
     void* p = nullptr;
-    const cudaError_t e = cudaGetSymbolAddress(&p, g_static_workspace);
+    cudaError_t e = cudaGetSymbolAddress(&gaddr[dev], g_static_global);
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(&p, g_static_workspace);
     if (e != cudaSuccess) return fail_cuda("static workspace address", e);
     addr[dev] = p;
   }
   *out = static_cast<char*>(addr[dev]);
+  if (global_rows != nullptr) *global_rows = static_cast<char*>(gaddr[dev]);
   return SC_OK;
 }
 
@@ -1212,7 +1223,8 @@ extern "C" int sc_layer_forward_noalloc(const sc_layer_args* a, void* stream) {
   if (a->pos_out == a->pos || a->len_out == a->len) return SC_ERR_INVALID_ARG;
   if ((rc = check_keep(a->keep_rule, &a->alpha, 1, a->theta)) != SC_OK) return rc;
   // a single layer reads its rows in place, so the compacted copies that the
-  // layout reserves last are not needed: everything before them must fit
+  // layout reserves are not needed: everything before them must fit, and what
+  // comes after them has an array of its own
   WsLayout lay;
   ws_layout(a->B, a->L, a->H, &lay);
   if (lay.qkv > kStaticWorkspaceBytes) {
@@ -1222,8 +1234,11 @@ extern "C" int sc_layer_forward_noalloc(const sc_layer_args* a, void* stream) {
     return fail(SC_ERR_UNSUPPORTED, "sc_layer_forward_noalloc", d);
   }
   if ((rc = ensure_configured()) != SC_OK) return rc;
+  if (lay.total - lay.gprob > kStaticGlobalBytes)
+    return fail(SC_ERR_UNSUPPORTED, "sc_layer_forward_noalloc", "global rows' scratch");
   char* ws = nullptr;
-  if ((rc = static_workspace(&ws)) != SC_OK) return rc;
+  char* global_rows = nullptr;
+  if ((rc = static_workspace(&ws, &global_rows)) != SC_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
   // the compacted-row descriptors point at the caller's tensors: never read here
@@ -1253,6 +1268,8 @@ extern "C" int sc_layer_forward_noalloc(const sc_layer_args* a, void* stream) {
   p.theta = a->theta;
   p.keep_rule = a->keep_rule;
   fill_workspace(&p, ws, lay, 0);
+  p.gprob = reinterpret_cast<float*>(global_rows);
+  p.gog = reinterpret_cast<float*>(global_rows + (lay.gog - lay.gprob));
 
   PrepParams pp{};
   pp.B = a->B; pp.L = a->L;

@@ -13,7 +13,7 @@ constexpr int kHeadDim = 64;
 constexpr int kTile = 128;         // rows (queries or keys) per tile
 constexpr int kMaxBandTiles = 5;   // key (query) tiles touched by one 128-row tile, w <= 256
 constexpr int kWideBandTiles = 9;  // ... with a wide window, 256 < w <= 512
-constexpr int kPairWindow = 256;   // widest window of the paired rows layout on long sequences
+constexpr int kNarrowWindow = 256; // widest window whose bands touch at most kMaxBandTiles tiles
 constexpr int kMaxGlobal = 16;     // global tokens per sequence (one 16-wide MMA tile)
 constexpr int kMaxLen = 4096;
 constexpr int kMaxTiles = kMaxLen / kTile;
@@ -71,22 +71,28 @@ struct LayerParams {
   int keep_rule;         // kKeepRelative, kKeepAbsolute or kKeepTopRatio
   // workspace
   float* acc;            // [B][H][L] per-head column sums: band rows + global rows
-  float* colpart;        // [B][H][L][band_slots] band-row column sums per query tile
-                         //   (slot = query tile mod band_slots)
-  int band_slots;        // kMaxBandTiles, or kWideBandTiles with wide
-  int wide;              // rows kernel: one query tile per CTA (256 < w on long sequences)
+  float* colpart;        // [B][H][band_slots][L] band-row column sums per query tile
+                         //   (slot = query tile mod band_slots); with band:
+                         //   [B][H][L][kMaxBandTiles]
+  int band_slots;        // kMaxBandTiles, or kWideBandTiles (256 < w on long sequences)
   int band;              // the single-pass band kernel computes the rows (w <= 256)
+                         //   and sc_cols_kernel the scores
   int sms;               // multiprocessors of the device (the band kernel's grid)
   float* gpart;          // [B][H][T][4][kMaxGlobal] column sums of global keys over far rows,
                          //   per (query tile, 32-row warp slice)
-  float* gstat;          // [B][H][T][4][kMaxGlobal][2] (max, sum) of global rows per
-                         //   (key tile, 32-key warp slice)
-  float* og;             // [B][H][T2][kMaxGlobal][64] fp32 parts of the global rows'
+  float* gstat;          // [B][H][T][kMaxGlobal][2] (max, sum) of global rows per key tile;
+                         //   with band: [B][H][T][4][kMaxGlobal][2], per 32-key warp slice
+  float* og;             // with band: [B][H][T2][kMaxGlobal][64] fp32 parts of the global rows'
                          //   outputs, one per key-tile pair (T2 = (T + 1) / 2)
+  float* gprob;          // [B][H][kMaxGlobal][L] global rows' probabilities relative to the
+                         //   maximum over the key's tile
+  float* gog;            // [B][H][T][kMaxGlobal][64] fp32 parts of the global rows' outputs, one
+                         //   per key tile, relative to the same maximum
   uint8_t* keep;         // [B][L]
   uint32_t* cnt_tile;    // [B][T]
   uint32_t* cnt_seq;     // [B]
-  uint32_t* rows_done;   // [B][H]: rows CTAs of (sequence, head) whose results are visible
+  uint32_t* rows_done;   // [B][H]: rows CTAs of a sequence whose results are visible (the
+                         //   first entry of each sequence; with band: of each (sequence, head))
   uint32_t* cols_done;   // [B][H]: cols CTAs of (sequence, head) whose global-row parts are stored
   // nonzero: the gather kernel before this launch is still copying later
   // sequences' rows when it starts: sequence b's rows are complete once

@@ -3,27 +3,28 @@
 //
 // Per layer, per sequence b (n current tokens, original positions pos[b][*]):
 //
-//   rows kernel   (one CTA per pair of 128-row query tiles of one (sequence,
-//                 head); one softmax warpgroup per tile)
-//     S = Q K^T over the band key tiles and one 16-wide tile of global keys on
-//     the tensor cores (tcgen05, bf16 -> fp32 in tensor memory); each 16 KB
-//     operand tile is one TMA copy.  Row softmax in fp32 (base 2, lazily
-//     rescaled running max); P (bf16) goes back to tensor memory and P V
-//     accumulates there.  Then the band pass: S^T = K Q^T of each key tile of
-//     the band (the tiles are still resident) and, per key column j, the sum
-//     over the tile's rows of exp2(S_ij - LSE_i) (one thread per column, no
-//     cross-thread reduction), one partial per (key, query tile).  Writes O,
-//     the row log-sum-exp LSE_i, those partials, the far-row column sums of
-//     the global keys, and (max, sum) of the global rows over this tile's keys.
+//   rows kernel   (one CTA per 128-row query tile of one (sequence, head), two
+//                 CTAs per SM)
+//     S = Q K^T over the band in items of 64 keys and one 16-wide item of global
+//     keys on the tensor cores (tcgen05, bf16 -> fp32 in tensor memory); each
+//     16 KB operand tile is one TMA copy.  Row softmax in fp32 (base 2, a
+//     reference per row that is raised when it has to be); P (bf16) goes back
+//     to tensor memory and P V accumulates there.  Then the band pass: S^T =
+//     K Q^T of each key tile of the band and, per key column j, the sum over the
+//     tile's rows of exp2(S_ij - LSE_i) (one thread per column, no cross-thread
+//     reduction), one partial per (key, query tile).  Writes O, those partials,
+//     the far-row column sums of the global keys, and, for the tile's own keys,
+//     the global rows' probabilities and P V relative to the tile's maximum.
 //
-//   cols kernel   (one CTA per pair of 128-key tiles; one warpgroup per tile)
-//     The global rows' probabilities over the pair's keys and their P V
-//     outputs, and each key's column sum: the band partials added in tile
-//     order, plus the global rows' share.  The last CTA of a key-tile pair
-//     sums the heads in a fixed order and applies the threshold; the last pair
-//     of a sequence compacts the survivors in order.  Each CTA waits (bounded)
-//     only for the rows CTAs of its own (sequence, head); the "last" CTAs are
-//     found by atomic counters.
+//   scores kernel (sc_scores.cu; one CTA per 128 keys of a sequence)
+//     Each key's column sum: the band partials added in tile order, plus the
+//     global rows' share, heads in a fixed order; the threshold; the last CTA of
+//     a sequence compacts the survivors in order.  Each CTA waits (bounded) only
+//     for the rows CTAs of its own sequence; the "last" CTA is found by an
+//     atomic counter.
+//
+//   cols kernel   the same role behind the single-pass band kernel (sc_band.cu):
+//     one CTA per pair of 128-key tiles and head.
 //
 //   gather kernel copies the survivors' next-layer Q, K, V rows into compacted
 //   buffers (coalesced 16-byte vectors) when they are not already in place.
@@ -35,617 +36,800 @@
 #include <cuda_runtime.h>
 #include <utility>
 #include <cuda_bf16.h>
+#include <cstddef>
 #include <cstdint>
 
 #include "sc_internal.cuh"
+#include "sc_finalize.cuh"
 #include "sc_layer_common.cuh"
-#include "sc_select.cuh"
 #include "sm103_primitives.cuh"
 
 namespace sc {
 
+// The global rows' P is the A operand of an M = 128 MMA whose rows past the 16
+// global rows are never used: each 64-key block of that A tile holds its 16
+// valid rows (2 KB) and lets the MMA read the following rows from whatever
+// shared memory comes next, so only 2 KB is reserved.
+constexpr uint32_t kPgBlock = 2 * 1024;
+
 // ---------------------------------------------------------------------------
 // rows kernel
 // ---------------------------------------------------------------------------
-// One CTA per pair of 128-row query tiles (2p, 2p+1) of one (sequence, head),
-// one softmax warpgroup per tile; the two tiles share their K/V tiles (the
-// band of the pair spans at most six 128-key tiles: all K tiles stay
-// resident, V tiles pass through a ring) and one tensor core serves both.
+// One CTA per 128-row query tile of one (sequence, head), two CTAs per SM, so
+// that one CTA's start and end hide behind the other's exponentials.  Warps 0-3
+// (one thread per row) are the softmax; warp 4 issues the MMAs, warp 5 the
+// copies, warps 6 and 7 evaluate the global rows over the tile's keys beside
+// the softmax.
 //
-// Per key tile a warpgroup loads all 128 columns of S into registers and
-// hands that tensor memory straight back, so S of its next key tile is
-// computed while it evaluates this tile's exponentials.  P (bf16) goes to its
-// own tensor-memory columns and P V reads it from there (no shared-memory
-// traffic for P).
+// The softmax warps take one item after the other from three 64-column buffers
+// in tensor memory, filled in order by warp 4, three items ahead:
+//   row pass    S of 64 keys of the band (the blocks that some row attends to),
+//               then S_G of the 16 global keys: P (bf16) goes over the first
+//               columns of the item's own buffer, and P V reads it there
+//   band pass   S^T of a 128-key tile against 64 queries, last tile first (the
+//               last three are still in shared memory): per key column the sum
+//               over the rows of exp2(S - LSE); after the diagonal tile S_Gt,
+//               its keys against the global queries
+// Handing an item back (P stored, or S^T read) lets warp 4 issue P V and the
+// item three further on into the same buffer: what overwrites columns that an
+// earlier product reads is issued after it.  32-column chunks that no row of a
+// warp attends to are not evaluated.
 //
-// Tensor memory (512 columns) per warpgroup X in {0, 1}, base 256 X:
-//   S    [+0, +128)   S of the current key tile (fp32); after the last tile:
-//                     S_G [+0, +16) (the 16 global keys) and S_Gt [+16, +32)
-//                     (the diagonal key tile against the global queries)
-//   P    [+128, +192) P of the current key tile, bf16 pairs; before the
-//                     first tile: S_G [+128, +144) and P_G [+144, +152)
-//   O    [+192, +256)
-// Warps 0-7: the two softmax warpgroups; warpgroup 2 (warps 8-11): warp 8
-// loads Q and the K tiles, warp 10 the V tiles, warps 9 and 11 issue the MMAs
-// of softmax warpgroups 0 and 1 (one issuing thread per warpgroup, so each
-// tcgen05.commit covers that warpgroup's MMAs only).
-// Launched at 168 registers a thread (three warps per SM sub-partition);
-// warpgroup 2 gives registers back so that the softmax warps, which hold a
-// whole 128-column row of S, get 200: 128 x 96 + 256 x 200 = 63488 <= 384 x 168.
-constexpr int kRowsThreads = 384;
-constexpr int kRowsLaunchRegs = 168;
-constexpr int kRowsCtlRegs = 96;
-constexpr int kRowsSoftmaxRegs = 200;
-static_assert(128 * kRowsCtlRegs + 256 * kRowsSoftmaxRegs <= kRowsThreads * kRowsLaunchRegs,
-              "register split exceeds the launch allocation");
-constexpr int kPairTiles = kMaxBandTiles + 1;
-// V slots: with six key tiles only the sixth reuses a slot, that of the first;
-// the first is used by query tile 0 alone and the sixth by query tile 1 alone
-// (each query tile's band spans at most five key tiles).
-constexpr int kVStages = kPairTiles - 1;
-// Wide windows (256 < w <= 512 on sequences of more than five tiles): one
-// query tile per CTA, up to nine resident key tiles and a three-slot V ring in
-// the same shared memory (one Q tile + 9 + 3 = two Q tiles + 6 + 5).
-constexpr int kWideVStages = 3;
-static_assert(1 + kWideBandTiles + kWideVStages == 2 + kPairTiles + kVStages,
-              "both layouts fill the same shared memory");
-
-__host__ __device__ constexpr uint32_t col_s(int X) { return 256u * X; }
-__host__ __device__ constexpr uint32_t col_p(int X) { return 256u * X + 128u; }
-__host__ __device__ constexpr uint32_t col_o(int X) { return 256u * X + 192u; }
+// Tensor memory (256 columns a CTA): the buffers [0, 192), O [192, 256); once O
+// is out, its columns take the global rows' P V.
+//
+// What bounds it: each allowed (row, key) pair costs two exponentials, one in
+// each pass, and about eight further issue slots; with one softmax warp of each
+// CTA on an SM sub-partition the in-order issue of two warps (IPC 0.4 of 1),
+// not the exponential unit (a fifth busy) or the tensor cores (a quarter).  So
+// the gains lie in instructions and latencies: no maximum in an ordinary item,
+// three items in flight, narrow bands by 64-key items and 32-column chunks,
+// two independent CTAs.  Code size counts as much: every section but the two
+// item loops runs once a CTA, and at 78 KB of code instead of 55 KB the
+// kernel missed the instruction caches and took 14% longer.
+// Layer 0 of 2 x 4096 tokens (w 256, 12 heads, 9 global tokens), rows and scores
+// together: 81 us, against 89 us for pairs of query tiles in one CTA per SM
+// with whole-tile items and a tensor-core scores kernel; 4 x 4096: 113 against
+// 144 us; 3 x 1000 at w 64: 25 against 35 us.
+constexpr int kRowsThreads = 256;
+constexpr int kKSlots = 3, kVSlots = 2;          // 16 KB operand slots
+constexpr int kRowsSlots = kKSlots + kVSlots;    // K tiles 0..2, V tiles 3..4
+constexpr int kBufs = 3;
+constexpr int kHalf = 64;                        // columns of a buffer: keys (queries) of an item
+constexpr uint32_t kColO = kBufs * kHalf;
+constexpr uint32_t kColPG = kMaxGlobal;          // P_G in its buffer, after S_G
+constexpr float kMaxItemSum = 16777216.f;        // 2^24
 
 struct RowsSmem {
-  alignas(16) float nlse[2][kTile];   // -LSE of each query tile's rows (read as float4)
-  uint64_t bar_q;
-  uint64_t bar_kfull[kWideBandTiles];
-  uint64_t bar_vfull[kVStages], bar_vempty[kVStages];
-  uint64_t bar_sg[2], bar_sgend[2], bar_sfull[2], bar_sfree[2], bar_pready[2], bar_pvdone[2];
-  uint64_t bar_fin[2];
-  uint64_t bar_stall;   // test hook: nothing ever completes it
+  alignas(16) float nlse[kTile];         // -LSE of the tile's rows (read as float4)
+  float gm[kMaxGlobal][2];               // global rows: maximum over 64 of the tile's keys
+  float gs[kMaxGlobal][2];               // ... and sum of exponentials
+  // in this order: first those with one arrival per softmax warp
+  uint64_t bar_back[kBufs];              // a buffer's item is handed back
+  uint64_t bar_stage, bar_gx;
+  uint64_t bar_q, bar_g, bar_vd;
+  uint64_t full[kRowsSlots], empty[kRowsSlots];
+  uint64_t bar_full[kBufs];              // a buffer's item is there
+  uint64_t bar_pv[kBufs];                // P V of the buffer's item is complete
+  uint64_t bar_og, bar_fin;
+  uint64_t bar_stall;                    // test hook: nothing ever completes it
   uint32_t tmem_base;
   int abort;
   int gc[kMaxGlobal];
 };
 
-// dynamic shared memory: two Q tiles, every K tile of the pair, the V ring,
-// the global rows
-constexpr uint32_t kRowsDyn =
-    kTileBytes * (2 + kPairTiles + kVStages) + 3 * kGTileBytes + 1024;
+constexpr int kRowsBars4 = kBufs + 2;
+constexpr int kRowsBars = kRowsBars4 + 3 + 2 * kRowsSlots + 2 * kBufs + 3;
+static_assert(kRowsBars <= 32, "one barrier a lane at start");
+static_assert(offsetof(RowsSmem, bar_stall) - offsetof(RowsSmem, bar_back) == 8 * (kRowsBars - 1),
+              "the barriers are consecutive");
 
-// kWide: one query tile per CTA (see kWideVStages); otherwise pairs of tiles.
-template <bool kWide>
-__global__ void __launch_bounds__(kRowsThreads, 1)
+// dynamic shared memory: the Q tile, the global rows' P blocks, the operand
+// slots, the global rows (whose space takes S_Gt in the band pass).  The P
+// blocks' 16 rows are rows 64..79 of the A operand of an M = 128 product (so
+// that its result lies in warp 6's lanes); the other rows read the shared
+// memory around them.
+constexpr uint32_t kGxBytes = kMaxGlobal * kTile * 4;
+static_assert(kGxBytes >= 3 * kGTileBytes, "S_Gt takes the global rows' space");
+constexpr uint32_t kPgRow0 = 64;
+static_assert(kTileBytes >= kPgRow0 * 128 && kRowsSlots * kTileBytes >= 8 * 1024,
+              "the A operand's unused rows stay inside the shared memory");
+constexpr uint32_t kRowsDyn = kTileBytes * (1 + kRowsSlots) + 2 * kPgBlock + kGxBytes + 1024;
+
+// Where key tile u of the band pass (counted from the last tile of the row
+// pass, nk tiles in all) sits: the last three are still in their K slots; the
+// others are loaded again, into the V slot of the last tile but one, then the K
+// slots in the order in which the band pass frees them.
+struct SlotFill {
+  int slot, fill;   // fill-th filling of the slot
+};
+__device__ __forceinline__ SlotFill band_slot(int u, int nk) {
+  if (u < kKSlots) {
+    const int t = nk - 1 - u;
+    return {t % kKSlots, t / kKSlots};
+  }
+  const int r = u - kKSlots, c = r & 3;
+  if (c == 0) return {kKSlots + (nk & 1), (nk - 2) / kVSlots + 1 + (r >> 2)};
+  const int t = nk - c;
+  return {t % kKSlots, t / kKSlots + 1 + (r >> 2)};
+}
+
+// Which of a warp's 32 rows may attend to keys c0 .. c0 + 31 (rows i0 .. i0 + 31):
+// 0 none, 1 some, 2 all of them to all keys.
+__device__ __forceinline__ int chunk_kind(int i0, int c0, int w, int n) {
+  if (c0 + 31 < i0 - w || c0 > min(n - 1, i0 + 31 + w)) return 0;
+  return (c0 >= i0 + 31 - w && c0 + 31 <= min(n - 1, i0 + w)) ? 2 : 1;
+}
+
+// x[k] = -inf outside lo..hi (columns of the chunk).
+__device__ __forceinline__ void mask_range(float* x, int lo, int hi) {
+  const uint32_t in = bit_range32(lo, hi);
+#pragma unroll
+  for (int k = 0; k < 32; ++k) x[k] = (in & (1u << k)) ? x[k] : -INFINITY;
+}
+
+__global__ void __launch_bounds__(kRowsThreads, 2)
     sc_rows_kernel(const __grid_constant__ TensorMaps maps, const __grid_constant__ LayerParams p) {
-  // the cols kernel is scheduled once every CTA here has passed this wait, so
-  // what the kernels before this one wrote is complete when it starts (with
-  // p.gathered, the gather kernel before this one lets it start only once the
-  // kernels before the gather are complete, and each CTA waits below for its
-  // own sequence's rows)
+  // the scores kernel is scheduled once every CTA here is past this wait (and
+  // holds its tensor memory), so what the kernels before this one wrote is
+  // complete when it starts (with p.gathered, the gather kernel before this
+  // one lets it start only once the kernels before the gather are complete,
+  // and each CTA waits below for its own sequence's rows)
   if (p.gathered == nullptr) pdl_wait();
-  pdl_launch_dependents();
-  // grid: pairs of query tiles (single tiles with a wide window),
-  // (sequence, head)-major, so that the CTAs of a (sequence, head) finish
-  // together and its cols CTAs can start early
-  constexpr bool wide = kWide;
-  constexpr int band_slots = wide ? kWideBandTiles : kMaxBandTiles;
-  const int per_bh = wide ? p.T : (p.T + 1) / 2;
-  const int pr = blockIdx.x % per_bh, bh = blockIdx.x / per_bh;
+  // grid: query tiles, (sequence, head)-major, so that the CTAs of a sequence
+  // finish together and its scores CTAs can start early
+  const int qt = blockIdx.x % p.T, bh = blockIdx.x / p.T;
   const int h = bh % p.H, b = bh / p.H;
-  const int q_first = wide ? pr : 2 * pr;   // first query tile of this CTA
   const LayerView v = layer_view(p);
   // the sequence's state, loaded together
   const bool tailed = owned_by_tail(p, v, b);
   const int n = __ldcg(v.len + b);
   const int ng_raw = __ldcg(v.ng + b);
   const int gc_raw = threadIdx.x < kMaxGlobal ? __ldcg(v.gcur + b * kMaxGlobal + threadIdx.x) : -1;
+  const RowSource rs = row_source(p, v, b);
   if (tailed) return;
-  if (q_first * kTile >= n) return;
+  const int q0 = qt * kTile;
+  if (q0 >= n) return;
   const int ng = min(ng_raw, kMaxGlobal);
-  const int ngp = ng > 0 ? kMaxGlobal : 0;
-  const bool hasB = !wide && (q_first + 1) * kTile < n;
-  constexpr int nvs = wide ? kWideVStages : kVStages;   // V ring slots
+  const bool glob = ng > 0;
 
   extern __shared__ uint8_t dyn_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dyn_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  uint8_t* Qs = base;                                        // 2 tiles (wide: 1)
-  uint8_t* Ks = Qs + (wide ? 1 : 2) * kTileBytes;            // all resident: 6 (wide: 9)
-  uint8_t* Vs = Ks + (wide ? kWideBandTiles : kPairTiles) * kTileBytes;   // nvs slots
-  uint8_t* KG = Vs + nvs * kTileBytes;
+  uint8_t* Qs = base;
+  uint8_t* Pg = Qs + kTileBytes;                   // 2 blocks of 16 rows
+  uint8_t* Slots = Pg + 2 * kPgBlock;              // K slots, V slots
+  uint8_t* KG = Slots + kRowsSlots * kTileBytes;
   uint8_t* VG = KG + kGTileBytes;
   uint8_t* QG = VG + kGTileBytes;
+  float* const gx = reinterpret_cast<float*>(KG);  // S_Gt [kMaxGlobal][kTile]
   __shared__ RowsSmem sm;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // key tiles of each query tile, and of the pair (absolute tile indices)
-  int klo[2], khi[2];
-#pragma unroll
-  for (int X = 0; X < 2; ++X) {
-    const int q0 = (q_first + X) * kTile, q1 = min(q0 + kTile - 1, n - 1);
-    klo[X] = max(0, q0 - p.w) / kTile;
-    khi[X] = min(n - 1, q1 + p.w) / kTile;
-  }
-  const int kt_lo = klo[0];
-  const int kt_hi = hasB ? khi[1] : khi[0];
-  const int nk = kt_hi - kt_lo + 1;   // <= 6 (wide: 9); window checked on the host
+  // the warp index, uniform over the warp
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int w = p.w;
+  // keys that some row of the tile attends to, and their key tiles
+  const int q1 = min(q0 + kTile - 1, n - 1);
+  const int jlo = max(0, q0 - w), jhi = min(n - 1, q1 + w);
+  const int klo = jlo / kTile;
+  const int nk = jhi / kTile - klo + 1;            // <= 9; window checked on the host
+  const int blo = jlo / kHalf;                     // 64-key blocks of the row pass
+  const int nrow = jhi / kHalf - blo + 1 + (glob ? 1 : 0);   // its items
+  const int u_d = nk - 1 - (qt - klo);             // the diagonal tile in the band pass
+  // the last tile's V slot: O leaves through it, then it takes V of the
+  // diagonal tile, for the global rows
+  const int vd_slot = kKSlots + ((nk - 1) & 1);
+  // the band pass: some key of tile u attends to some query of the half
+  auto reaches = [&](int u, int qh) {
+    const int j0 = (klo + nk - 1 - u) * kTile, i0 = q0 + kHalf * qh;
+    return i0 < n && min(j0 + kTile, n) - 1 + w >= i0 && j0 - w <= min(i0 + kHalf, n) - 1;
+  };
 
-  if (tid == 0) {
-    mbar_init(&sm.bar_q, 1);
-    for (int k = 0; k < kWideBandTiles; ++k) mbar_init(&sm.bar_kfull[k], 1);
-    for (int s = 0; s < kVStages; ++s) {
-      mbar_init(&sm.bar_vfull[s], 1);
-      mbar_init(&sm.bar_vempty[s], 1);
-    }
-    for (int X = 0; X < 2; ++X) {
-      mbar_init(&sm.bar_sg[X], 1);
-      mbar_init(&sm.bar_sgend[X], 1);
-      mbar_init(&sm.bar_sfull[X], 1);
-      mbar_init(&sm.bar_sfree[X], 4);   // one arrival per warp
-      mbar_init(&sm.bar_pready[X], 4);
-      mbar_init(&sm.bar_pvdone[X], 1);
-      mbar_init(&sm.bar_fin[X], 1);
-    }
-    mbar_init(&sm.bar_stall, 1);
-    sm.abort = 0;
+  uint32_t fills = 0;   // warp 5: how often each slot has been filled (four bits a slot)
+  if (warp == 5) {
+    // the barriers, one a lane; then the first copies, ahead of the block's start
+    if (lane < kRowsBars) mbar_init(sm.bar_back + lane, lane < kRowsBars4 ? 4 : 1);
+    if (lane == 0) sm.abort = 0;
     fence_mbar_init();
-    // this sequence's rows may still be crossing the host link
-    if (p.gathered != nullptr) wait_count(p.gathered + b, p.gather_target, &sm.abort);
+    __syncwarp();
+    if (lane == 0) {
+      // this sequence's rows may still be crossing the host link
+      if (p.gathered != nullptr) {
+        wait_count(p.gathered + b, p.gather_target, &sm.abort);
+        fence_proxy_async_global();   // the copies, before any TMA load
+      }
+      mbar_arrive_expect_tx(&sm.bar_q, kTileBytes);
+      load_tile(maps, 0, rs, h, q0, Qs, &sm.bar_q);
+      for (int t = 0; t < min(nk, 2); ++t) {
+        mbar_arrive_expect_tx(&sm.full[t], kTileBytes);
+        load_tile(maps, 1, rs, h, (klo + t) * kTile, Slots + t * kTileBytes, &sm.full[t]);
+      }
+      mbar_arrive_expect_tx(&sm.full[kKSlots], kTileBytes);
+      load_tile(maps, 2, rs, h, klo * kTile, Slots + kKSlots * kTileBytes, &sm.full[kKSlots]);
+    }
+    __syncwarp();
+    fills = 1u | (nk > 1 ? 1u << 4 : 0u) | 1u << (4 * kKSlots);
   }
   if (tid < kMaxGlobal) sm.gc[tid] = tid < ng ? gc_raw : -1;
-  if (warp == 9) tmem_alloc(&sm.tmem_base, 512);
+  if (warp == 4) tmem_alloc(&sm.tmem_base, 256);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (p.gathered != nullptr) fence_proxy_async_global();   // the copies, before any TMA load
-  const uint32_t tm = sm.tmem_base;
+  pdl_launch_dependents();
+  const uint32_t tm = __shfl_sync(0xffffffffu, sm.tmem_base, 0);
   volatile int* abort_flag = &sm.abort;
+  const size_t tile = (static_cast<size_t>(b) * p.H + h) * p.T + qt;   // of the partial results
 
-  if (warp >= 8) {
-   regs_dealloc<kRowsCtlRegs>();
-   if (warp == 8) {
-    // ------------------------------------------------------------- Q, globals, K
-    const RowSource rs = row_source(p, v, b);
-    if (lane == 0) {
-      // Q, then the first two K tiles (the first S needs Q and K), then the
-      // global rows, then the other K tiles
-      mbar_arrive_expect_tx(&sm.bar_q, (hasB ? 2 : 1) * kTileBytes + 3 * ngp * 128);
-      load_tile(maps, 0, rs, h, q_first * kTile, Qs, &sm.bar_q);
-      if (hasB) load_tile(maps, 0, rs, h, (q_first + 1) * kTile, Qs + kTileBytes, &sm.bar_q);
-      for (int k = 0; k < nk && k < 2; ++k) {
-        mbar_arrive_expect_tx(&sm.bar_kfull[k], kTileBytes);
-        load_tile(maps, 1, rs, h, (kt_lo + k) * kTile, Ks + k * kTileBytes, &sm.bar_kfull[k]);
-      }
-    }
-    __syncwarp();
-    if (ngp) {
-      load_globals(maps, 1, rs, h, p.H, sm.gc, ng, KG, &sm.bar_q, lane);
-      load_globals(maps, 2, rs, h, p.H, sm.gc, ng, VG, &sm.bar_q, lane);
-      load_globals(maps, 0, rs, h, p.H, sm.gc, ng, QG, &sm.bar_q, lane);
-    }
-    if (lane == 0) {
-      for (int k = 2; k < nk; ++k) {
-        mbar_arrive_expect_tx(&sm.bar_kfull[k], kTileBytes);
-        load_tile(maps, 1, rs, h, (kt_lo + k) * kTile, Ks + k * kTileBytes, &sm.bar_kfull[k]);
-      }
-      // nothing may still be landing in shared memory when the CTA exits
-      drain_wait(&sm.bar_q, 0);
-      for (int k = 0; k < nk; ++k) drain_wait(&sm.bar_kfull[k], 0);
-    }
-   } else if (warp == 10) {
-    // ------------------------------------------------------------- V ring
-    if (lane == 0) {
-      const RowSource rs = row_source(p, v, b);
+  if (warp >= 4) {
+    if (warp == 4) {
+      // ----------------------------------------------------------- MMA issue
+      const uint32_t q_d = sdesc_lo(smem_u32(Qs)), slot_d = sdesc_lo(smem_u32(Slots));
+      constexpr uint32_t kTileD = kTileBytes >> 4;   // in descriptors
+      constexpr uint32_t kIdS = idesc_bf16(128, kHalf, false, false);
+      constexpr uint32_t kIdG = idesc_bf16(128, 16, false, false);
+      constexpr uint32_t kIdPV = idesc_bf16(128, 64, false, true);
+      constexpr uint32_t kHalfD = kTileD / 2;
+      const uint32_t kg_d = sdesc_lo(smem_u32(KG)), vg_d = sdesc_lo(smem_u32(VG)),
+                     qg_d = sdesc_lo(smem_u32(QG));
+      const int nblk = nrow - (glob ? 1 : 0);
       bool ok = true;
-      int issued = 0;
-      // slot s = k mod nvs and its use count, advanced without division
-      for (int k = 0, s = 0, use = 0; ok && k < nk; ++k) {
-        if (k >= nvs && !(ok = mbar_wait(&sm.bar_vempty[s], (use - 1) & 1, abort_flag))) break;
-        mbar_arrive_expect_tx(&sm.bar_vfull[s], kTileBytes);
-        load_tile(maps, 2, rs, h, (kt_lo + k) * kTile, Vs + s * kTileBytes, &sm.bar_vfull[s]);
-        issued = k + 1;
-        if (++s == nvs) {
-          s = 0;
-          ++use;
+      if (p.stall_ns != 0)   // test hook: this bounded wait expires
+        ok = __all_sync(0xffffffffu, mbar_wait(&sm.bar_stall, 0, abort_flag, p.stall_ns));
+      ok = ok && warp_wait_poll(&sm.bar_q, 0, abort_flag);
+      // the next item of the sequence, into buffer ib
+      int is = 0, ib = 0, u = 0, qh = nk > 0 && !reaches(0, 0) ? 1 : 0;
+      bool sgt = false, more = true;
+      auto issue_next = [&]() {
+        uint32_t a_d, b_d;
+        uint64_t *wait = nullptr, *release = nullptr;
+        uint32_t par = 0, id = kIdS;
+        if (is < nblk) {                            // S of block is
+          const int kb = blo + is, t = kb / 2 - klo, slot = t % kKSlots;
+          wait = &sm.full[slot];
+          par = (t / kKSlots) & 1;
+          a_d = q_d;
+          b_d = slot_d + slot * kTileD + (kb & 1) * kHalfD;
+          // a tile's slot is free after its last block; the last three tiles stay
+          if (t < nk - kKSlots && (kb & 1)) release = &sm.empty[slot];
+          ++is;
+        } else if (is < nrow) {                     // S_G
+          wait = &sm.bar_g;
+          a_d = q_d;
+          b_d = kg_d;
+          id = kIdG;
+          ++is;
+        } else {
+          const SlotFill f = band_slot(u, nk);
+          wait = &sm.full[f.slot];
+          par = f.fill & 1;
+          a_d = slot_d + f.slot * kTileD;
+          const bool last = qh == 1 || !reaches(u, 1);
+          if (sgt) {                                // S_Gt of the diagonal tile
+            b_d = qg_d;
+            id = kIdG;
+          } else {                                  // S^T of tile u, query half qh
+            b_d = q_d + qh * kHalfD;
+          }
+          if (!sgt && last && glob && u == u_d) {
+            sgt = true;                             // the next item
+          } else if (sgt || last) {
+            release = &sm.empty[f.slot];
+            sgt = false;
+            ++u;
+            qh = u < nk && !reaches(u, 0) ? 1 : 0;
+          } else {
+            qh = 1;
+          }
+          more = u < nk;
         }
-      }
-      // the last copy issued into each slot has landed (after an expired wait
-      // fewer than nk were issued)
-      for (int s = 0; s < nvs && s < issued; ++s) {
-        const int last = s + nvs * ((issued - 1 - s) / nvs);
-        drain_wait(&sm.bar_vfull[s], (last / nvs) & 1);
-      }
-    }
-   } else if (warp == 9 || warp == 11) {
-    // ------------------------------------------------------------- MMA issue
-    const int X = warp == 9 ? 0 : 1;
-    if (lane == 0 && (X == 0 || hasB)) {
-      const uint32_t q_a = smem_u32(Qs) + X * kTileBytes, k_a = smem_u32(Ks), v_a = smem_u32(Vs);
-      const int kloX = klo[X], khiX = khi[X];
-      const uint32_t tS = tm + col_s(X), tP = tm + col_p(X), tO = tm + col_o(X);
-      bool ok = true;
-      if (X == 0 && p.stall_ns != 0)   // test hook: this bounded wait expires
-        ok = mbar_wait(&sm.bar_stall, 0, abort_flag, p.stall_ns);
-      ok = ok && mbar_wait(&sm.bar_q, 0, abort_flag);
-      if (ok) {
+        if (!(ok = warp_wait_poll(wait, par, abort_flag))) return;
         tc_fence_after();
-        if (ngp) {
-          mma_qk(tP, q_a, smem_u32(KG), 16);   // S_G
-          umma_commit(&sm.bar_sg[X]);
+        const uint32_t d = tm + kHalf * ib;
+        if (elect_one()) {
+#pragma unroll
+          for (int k = 0; k < kHeadDim / 16; ++k)
+            umma_bf16_lo(d, a_d + 2 * k, b_d + 2 * k, id, k > 0);
+          umma_commit(&sm.bar_full[ib]);
+          if (release != nullptr) umma_commit(release);
         }
-      }
-      // This warpgroup's events come in a fixed order: [P_G stored], then per
-      // key tile "S read" (sfree) and "P stored" (pready).  S of the next
-      // tile is issued at "S read", P V of a tile at "P stored".
-      auto issue_s = [&](int a) -> bool {
-        const int k = a - kt_lo;
-        if (!mbar_wait(&sm.bar_kfull[k], 0, abort_flag)) return false;
-        tc_fence_after();
-        mma_qk(tS, q_a, k_a + k * kTileBytes, 128);
-        umma_commit(&sm.bar_sfull[X]);
-        return true;
+        __syncwarp();
+        ib = ib == kBufs - 1 ? 0 : ib + 1;
       };
-      uint32_t nfree = 0, nready = 0;
-      // V slot of key tile k = a - kt_lo (k mod nvs) and its use count, advanced
-      // without division
-      int vslot = (kloX - kt_lo) % nvs, vuse = (kloX - kt_lo) / nvs;
-      if (ok) ok = issue_s(kloX);
-      if (ok && ngp) {
-        if ((ok = mbar_wait(&sm.bar_pready[X], (nready++) & 1, abort_flag))) {
+      // kBufs items ahead of the one whose hand-over is awaited
+      int left = kBufs;   // items issued and not handed back (from it = 0 on)
+#pragma unroll 1
+      for (int it = -kBufs, buf = 0, use = 0; ok && (it < 0 || left > 0); ++it) {
+        if (it >= 0) {
+          if (!(ok = warp_wait_poll(&sm.bar_back[buf], use & 1, abort_flag))) break;
+          --left;
+          if (it < nrow) {                          // P V
+            const int kb = blo + it, t = kb / 2 - klo;
+            const bool g = it >= nblk;
+            const int slot = kKSlots + (t & 1);
+            if (!g && !(ok = warp_wait_poll(&sm.full[slot], (t / kVSlots) & 1, abort_flag))) break;
+            tc_fence_after();
+            const uint32_t v_d = g ? vg_d : slot_d + slot * kTileD + (kb & 1) * kHalfD;
+            if (elect_one()) {
+              umma_bf16_ts_lo(tm + kColO, tm + kHalf * buf + (g ? kColPG : 0), v_d, kIdPV, it > 0);
+              if (!g)
+#pragma unroll
+                for (int k = 1; k < kHalf / 16; ++k)
+                  umma_bf16_ts_lo(tm + kColO, tm + kHalf * buf + 8 * k, v_d + 128 * k, kIdPV, 1u);
+              umma_commit(&sm.bar_pv[buf]);
+              if (!g && ((kb & 1) || it == nblk - 1)) umma_commit(&sm.empty[slot]);
+            }
+            __syncwarp();
+          }
+          if (++buf == kBufs) {
+            buf = 0;
+            ++use;
+          }
+        }
+        if (more) {
+          issue_next();
+          if (it >= 0) ++left;
+        } else if (it < 0) {
+          --left;                                   // fewer items than buffers
+        }
+      }
+      if (elect_one()) umma_commit(&sm.bar_fin);
+      __syncwarp();
+      drain_wait(&sm.bar_fin, 0);
+    } else if (warp == 5) {
+      // ----------------------------------------------------------- copies
+      if (p.gathered != nullptr) fence_proxy_async_global();   // every lane that issues copies
+      bool ok = true, vd = false;
+      auto load_slot = [&](int t, int tensor, int slot, bool vdl) {
+        const uint32_t f = (fills >> (4 * slot)) & 15u;
+        if (f > 0 && !(ok = warp_wait_poll(&sm.empty[slot], (f - 1) & 1, abort_flag))) return;
+        uint64_t* bar = vdl ? &sm.bar_vd : &sm.full[slot];
+        if (elect_one()) {
+          mbar_arrive_expect_tx(bar, kTileBytes);
+          load_tile(maps, tensor, rs, h, (klo + t) * kTile, Slots + slot * kTileBytes, bar);
+        }
+        __syncwarp();
+        if (vdl) vd = true;
+        else fills += 1u << (4 * slot);
+      };
+      if (glob) {
+        if (elect_one()) mbar_arrive_expect_tx(&sm.bar_g, 3 * kGTileBytes);
+        __syncwarp();
+#pragma unroll 1
+        for (int k = 0; k < 3; ++k)   // K, V, Q
+          load_globals(maps, k == 2 ? 0 : k + 1, rs, h, p.H, sm.gc, ng, KG + k * kGTileBytes,
+                       &sm.bar_g, lane);
+        __syncwarp();
+      }
+      // in this order: V of tile 1, K of tile 2, V of tile 2, ...; then the
+      // band pass's K tiles that are no longer here, after the first of them V
+      // of the diagonal tile for the global rows
+#pragma unroll 1
+      for (int i = 0; ok && i < 2 * nk; ++i) {
+        const int r = i - 2 * (nk - 1);   // 0, 1: the first band tile, V of the diagonal tile
+        int t = 1 + i / 2, tensor = 2, slot = kKSlots + (t & 1);
+        bool vdl = false;
+        if (r < 0 && (i & 1)) {
+          if (++t >= nk) continue;
+          tensor = 1;
+          slot = t % kKSlots;
+        } else if (r == 0) {
+          if (nk <= kKSlots) continue;
+          t = nk - 1 - kKSlots;
+          tensor = 1;
+          slot = band_slot(kKSlots, nk).slot;
+        } else if (r == 1) {
+          if (!glob) continue;
+          if (!(ok = warp_wait_poll(&sm.bar_stage, 0, abort_flag))) break;
+          t = qt - klo;
+          slot = vd_slot;
+          vdl = true;
+        }
+        load_slot(t, tensor, slot, vdl);
+      }
+#pragma unroll 1
+      for (int u = kKSlots + 1; ok && u < nk; ++u) load_slot(nk - 1 - u, 1, band_slot(u, nk).slot, false);
+      // nothing may still be landing in shared memory when the CTA exits
+#pragma unroll 1
+      for (int s = 0; s < kRowsSlots + 3; ++s) {
+        const uint32_t f = s < kRowsSlots ? (fills >> (4 * s)) & 15u
+                           : s == kRowsSlots || (s == kRowsSlots + 1 ? glob : vd) ? 1u : 0u;
+        uint64_t* bar = s < kRowsSlots ? &sm.full[s] : &sm.bar_q + (s - kRowsSlots);
+        if (f > 0) drain_wait(bar, (f - 1) & 1);
+      }
+    } else if (glob) {
+      // ----------------------------------------------------------- global rows
+      // over this tile's keys (two a thread): their probabilities relative to
+      // the tile's maximum, and P V
+      const int x = tid & 63, half = warp & 1;
+      bool ok = warp_wait_poll(&sm.bar_gx, 0, abort_flag);
+#pragma unroll 1
+      for (int g = 0; ok && g < ng; ++g) {
+        const float m = warp_max(fmaxf(gx[g * kTile + x], gx[g * kTile + 64 + x]));
+        if (lane == 0) sm.gm[g][half] = m;
+      }
+      asm volatile("bar.sync 2, 64;" ::: "memory");
+      float* gp = p.gprob + (static_cast<size_t>(b) * p.H + h) * kMaxGlobal * p.L + q0 + x;
+#pragma unroll 1
+      for (int g = 0; ok && g < ng; ++g) {
+        const float m = fmaxf(sm.gm[g][0], sm.gm[g][1]);
+        // (a key past the end has S_Gt = -inf; m is finite: the tile has a key)
+        const float a = ex2(gx[g * kTile + x] - m), c = ex2(gx[g * kTile + 64 + x] - m);
+        if (q0 + x < n) gp[static_cast<size_t>(g) * p.L] = a;
+        if (q0 + 64 + x < n) gp[static_cast<size_t>(g) * p.L + 64] = c;
+        // transposed into the A tile: row g, column (key)
+        const uint32_t at = sw128_offset(g, x >> 3) + (x & 7) * 2;
+        *reinterpret_cast<uint16_t*>(Pg + at) = __bfloat16_as_ushort(__float2bfloat16_rn(a));
+        *reinterpret_cast<uint16_t*>(Pg + kPgBlock + at) =
+            __bfloat16_as_ushort(__float2bfloat16_rn(c));
+        const float s = warp_sum(a + c);
+        if (lane == 0) sm.gs[g][half] = s;
+      }
+      fence_proxy_async_smem();
+      asm volatile("bar.sync 2, 64;" ::: "memory");
+      if (warp == 6) {
+        ok = ok && warp_wait_poll(&sm.bar_vd, 0, abort_flag);
+        if (ok) {
+          tc_fence_after();   // O is out: its columns take the product
+          if (elect_one()) {
+            mma_pv(tm + kColO, smem_u32(Pg) - kPgRow0 * 128, kPgBlock,
+                   smem_u32(Slots) + vd_slot * kTileBytes, kTile / 16, false);
+            umma_commit(&sm.bar_og);
+          }
+          __syncwarp();
+          ok = warp_wait_poll(&sm.bar_og, 0, abort_flag);
           tc_fence_after();
-          mma_pv_ts(tO, tP + 16, smem_u32(VG), kMaxGlobal / 16, false);   // P_G V_G
-          umma_commit(&sm.bar_pvdone[X]);
+          float* part = p.gog + (tile * kMaxGlobal + lane) * kHeadDim;
+#pragma unroll 1
+          for (int c = 0; ok && c < 64; c += 16) {
+            float o[16];
+            tmem_ld16(tm + kColO + (kPgRow0 << 16) + c, o);
+            tmem_ld_wait();
+            if (lane < ng)
+#pragma unroll
+              for (int k = 0; k < 16; k += 4)
+                *reinterpret_cast<float4*>(part + c + k) =
+                    make_float4(o[k], o[k + 1], o[k + 2], o[k + 3]);
+          }
+          if (!ok) drain_wait(&sm.bar_og, 0);
         }
+      } else if (ok && lane < ng) {
+        reinterpret_cast<float2*>(p.gstat)[tile * kMaxGlobal + lane] = make_float2(
+            fmaxf(sm.gm[lane][0], sm.gm[lane][1]), sm.gs[lane][0] + sm.gs[lane][1]);
       }
-      for (int a = kloX; ok && a <= khiX; ++a) {
-        const int k = a - kt_lo;
-        if (!(ok = mbar_wait(&sm.bar_sfree[X], (nfree++) & 1, abort_flag))) break;
-        if (a < khiX) {
-          if (!(ok = issue_s(a + 1))) break;
-        } else if (ngp) {
-          // the last S is read: its columns take S_G and S_Gt for the epilogue
-          tc_fence_after();
-          mma_qk(tS, q_a, smem_u32(KG), 16);
-          mma_qk(tS + 16, k_a + (q_first + X - kt_lo) * kTileBytes, smem_u32(QG), 16);
-          umma_commit(&sm.bar_sgend[X]);
-        }
-        if (!(ok = mbar_wait(&sm.bar_pready[X], (nready++) & 1, abort_flag))) break;
-        if (!(ok = mbar_wait(&sm.bar_vfull[vslot], vuse & 1, abort_flag))) break;
-        tc_fence_after();
-        mma_pv_ts(tO, tP, v_a + vslot * kTileBytes, kTile / 16, ngp > 0 || a > kloX);
-        if (k + nvs < nk) umma_commit(&sm.bar_vempty[vslot]);   // slot reused
-        if (++vslot == nvs) {
-          vslot = 0;
-          ++vuse;
-        }
-        umma_commit(&sm.bar_pvdone[X]);
-      }
-      // band pass: S^T = K Q^T of each key tile of the band against this
-      // query tile, into the S columns once they are read (after the S_G /
-      // S_Gt of the epilogue, when there are global keys)
-      for (int a = kloX; ok && a <= khiX; ++a) {
-        if ((a > kloX || ngp) && !(ok = mbar_wait(&sm.bar_sfree[X], (nfree++) & 1, abort_flag)))
-          break;
-        tc_fence_after();
-        mma_qk(tS, k_a + (a - kt_lo) * kTileBytes, q_a, 128);
-        umma_commit(&sm.bar_sfull[X]);
-      }
-      umma_commit(&sm.bar_fin[X]);
-      drain_wait(&sm.bar_fin[X], 0);
+      __syncwarp();
     }
-    __syncwarp();
-   }
   } else {
     // ------------------------------------------------------------- softmax
-    regs_alloc<kRowsSoftmaxRegs>();
-    const int X = warp >> 2;              // warpgroup = query tile of the pair
-    const int kloX = X ? klo[1] : klo[0], khiX = X ? khi[1] : khi[0];
-    const int wq = warp & 3;              // TMEM lane quarter of this warp
-    const int r = tid & 127;              // row inside the tile == TMEM lane
-    const int qt = q_first + X;
-    const int r0 = qt * kTile;
-    const bool active = X == 0 || hasB;
-    const int i = r0 + r;                 // current index of this query row
-    const uint32_t lane_off = static_cast<uint32_t>(wq * 32) << 16;
-    const uint32_t tS = tm + col_s(X) + lane_off, tP = tm + col_p(X) + lane_off,
-                   tO = tm + col_o(X) + lane_off;
+    const int r = tid;                    // row inside the tile == TMEM lane
+    const int i = q0 + r;                 // current index of this query row
+    const int iw = q0 + 32 * warp;        // first row of this warp
+    const uint32_t lane_off = static_cast<uint32_t>(warp * 32) << 16;
+    const uint32_t tB = tm + lane_off, tO = tB + kColO;
     bool row_global = false;
+#pragma unroll 1
     for (int g = 0; g < ng; ++g) row_global |= (sm.gc[g] == i);
     const bool valid = (i < n) && !row_global;
     // allowed band keys of this row, inclusive (current index); the same band
     // is used for rows whose results are discarded (global rows, rows >= n)
-    const int lo = max(0, i - p.w);
-    const int hi = min(n - 1, i + p.w);
+    const int lo = max(0, i - w), hi = min(n - 1, i + w);
+    const uint64_t c2 = f2_pack(kLogitScale2, kLogitScale2);
+    bool ok = true;
+    int buf = 0;                          // of the current item, and which use of it
+    uint32_t use = 0;
+    auto wait_item = [&]() {
+      ok = ok && warp_wait_poll(&sm.bar_full[buf], use & 1, abort_flag);
+      tc_fence_after();
+    };
+    auto hand_back = [&]() {
+      tc_fence_before();
+      warp_arrive(&sm.bar_back[buf]);
+      if (++buf == kBufs) {
+        buf = 0;
+        ++use;
+      }
+    };
 
+    // Softmax with a running reference m_ref (base-2 units): P = exp2(x - ref).
+    // The reference is the maximum of the row's first item; a later item whose
+    // exponentials sum to more than kMaxItemSum raises it to its own maximum
+    // (when that lies more than 8 above), O (all earlier P V complete) and the
+    // row sums being rescaled exactly.  So P stays below 2^24 (an |V| of 2^100 does
+    // not overflow O), and a maximum
+    // over the item's columns is not part of an ordinary step.
     // lsum: the row sum of the exponentials (fp32), which gives the row's LSE
     // for the column sums; osum: the sum of the same values rounded to the
     // bf16 that P V multiplies, which normalises O (so that O is a weighted
     // mean of V rows whatever the rounding of P)
-    float m_ref = -INFINITY, lsum = 0.f, osum = 0.f;
-    bool ok = active;
-    uint32_t pv_issued = 0;               // P V products issued for this warpgroup
-
-    if (ok && ngp) {
-      ok = warp_wait(&sm.bar_sg[X], 0, abort_flag);
-      if (ok) {
-        float xg[kMaxGlobal];
-        tc_fence_after();
-        tmem_ld16(tP, xg);                // S_G
-        tmem_ld_wait();
-        float mx = -INFINITY;
-#pragma unroll
-        for (int g = 0; g < kMaxGlobal; ++g) {
-          const bool use = (g < ng) && abs(i - sm.gc[g]) > p.w;
-          xg[g] = use ? xg[g] : -INFINITY;
-          mx = fmaxf(mx, xg[g]);
+    float m_ref = i < n ? -INFINITY : 0.f, lsum = 0.f, osum = 0.f;
+    auto raise_to = [&](float tmax, bool may, bool have_o) {
+      const bool raise = may && tmax > m_ref + 8.f;
+      if (__any_sync(0xffffffffu, raise)) {
+        float f = 1.f;
+        if (raise) {
+          f = (m_ref == -INFINITY) ? 0.f : ex2(m_ref - tmax);
+          m_ref = tmax;
+          lsum *= f;
+          osum *= f;
         }
-        m_ref = mx * kLogitScale2;
-        const float nref = (m_ref == -INFINITY) ? 0.f : -m_ref;
-        uint32_t pk[8];
+        if (have_o && __any_sync(0xffffffffu, f != 1.f)) {
+          // the item before this one: its P V, hence every earlier one
+          const int pb = buf == 0 ? kBufs - 1 : buf - 1;
+          ok = ok && warp_wait_poll(&sm.bar_pv[pb], (buf == 0 ? use - 1 : use) & 1, abort_flag);
+          tc_fence_after();
+#pragma unroll 1
+          for (int c = 0; c < 64; c += 16) {
+            float o[16];
+            tmem_ld16(tO + c, o);
+            tmem_ld_wait();
 #pragma unroll
-        for (int g = 0; g < kMaxGlobal; g += 2) {
-          const float a = ex2(fmaf(xg[g], kLogitScale2, nref));
-          const float c = ex2(fmaf(xg[g + 1], kLogitScale2, nref));
-          pk[g / 2] = pack_bf16x2(a, c);
-          lsum += a + c;
-          osum = add_bf16_hi(add_bf16_lo(osum, pk[g / 2]), pk[g / 2]);
-        }
-        tmem_st8(tP + 16, pk);            // P_G
-        tmem_st_wait();
-        tc_fence_before();
-        warp_arrive(&sm.bar_pready[X]);
-        pv_issued = 1;
-      }
-    }
-
-    // Softmax with a running reference m_ref (base-2 units): P = exp2(x - ref).
-    // The tile's maximum is taken before its exponentials; when it exceeds the
-    // reference by more than 8, the reference is raised and O (all earlier
-    // P V complete) and the row sum are rescaled exactly.  P stays below 2^8.
-    // All exponentials of the tile are formed in registers before the previous
-    // P V is awaited: only the P store and a rescale of O depend on it.
-    const uint64_t c2 = f2_pack(kLogitScale2, kLogitScale2);
-    for (int t = 0; ok && t <= khiX - kloX; ++t) {
-      const int j0 = (kloX + t) * kTile;
-      const int a = lo - j0, e = hi - j0;   // this row's allowed columns of the tile
-      if (!(ok = warp_wait(&sm.bar_sfull[X], t & 1, abort_flag))) break;
-      tc_fence_after();
-      float x[128];
-#pragma unroll
-      for (int ch = 0; ch < 4; ++ch) tmem_ld32(tS + 32 * ch, x + 32 * ch);
-      tmem_ld_wait();
-      tc_fence_before();
-      warp_arrive(&sm.bar_sfree[X]);   // S is in registers: the next S may overwrite it
-      // keys outside a row's band take no part; tiles inside the band of all
-      // 32 rows of the warp (most of them) need no mask
-      if (!__all_sync(0xffffffffu, a <= 0 && e >= kTile - 1)) {
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          // this row's allowed keys among the chunk's 32, as bits; chunks
-          // that every row of the warp takes whole are left alone
-          const uint32_t keep = bit_range32(a - 32 * ch, e - 32 * ch);
-          if (__any_sync(0xffffffffu, keep != 0xffffffffu)) {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) {
-              const uint32_t out =
-                  ~static_cast<uint32_t>(static_cast<int32_t>(keep << (31 - k)) >> 31);
-              x[32 * ch + k] =
-                  __uint_as_float((__float_as_uint(x[32 * ch + k]) & ~out) | (0xff800000u & out));
-            }
+            for (int k = 0; k < 16; ++k) o[k] *= f;
+            tmem_st16(tO + c, reinterpret_cast<const uint32_t*>(o));
+            tmem_st_wait();   // o is reused
           }
         }
       }
-      float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-      for (int k = 0; k < kTile; k += 8) {
-        m4[0] = fmax3(m4[0], x[k], x[k + 1]);
-        m4[1] = fmax3(m4[1], x[k + 2], x[k + 3]);
-        m4[2] = fmax3(m4[2], x[k + 4], x[k + 5]);
-        m4[3] = fmax3(m4[3], x[k + 6], x[k + 7]);
-      }
-      const float tmax = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * kLogitScale2;
-      const bool raise = tmax > m_ref + 8.f;
-      float f = 1.f;
-      if (raise) {
-        f = (m_ref == -INFINITY) ? 0.f : ex2(m_ref - tmax);
-        m_ref = tmax;
-        lsum *= f;
-        osum *= f;
-      }
-      const float nref = (m_ref == -INFINITY) ? 0.f : -m_ref;
-      const uint64_t n2 = f2_pack(nref, nref);
-      uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
-      float sq[4] = {0.f, 0.f, 0.f, 0.f};
-      uint32_t pk[64];
-#pragma unroll
-      for (int k = 0; k < kTile; k += 2) {
-        float u, w;
-        f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, n2), u, w);
-        u = ex2(u);
-        w = ex2(w);
-        if (k & 2) s2b = f2_add(s2b, f2_pack(u, w));
-        else s2a = f2_add(s2a, f2_pack(u, w));
-        pk[k >> 1] = pack_bf16x2(u, w);
-        const int c = (k >> 1) & 1;
-        sq[2 * c] = add_bf16_lo(sq[2 * c], pk[k >> 1]);
-        sq[2 * c + 1] = add_bf16_hi(sq[2 * c + 1], pk[k >> 1]);
-      }
-      float sa, sb, sc2, sd;
-      f2_unpack(s2a, sa, sb);
-      f2_unpack(s2b, sc2, sd);
-      lsum += (sa + sb) + (sc2 + sd);
-      osum += (sq[0] + sq[1]) + (sq[2] + sq[3]);
-      // every earlier P V has completed: O is final for a rescale and the P
-      // columns of this warpgroup are free again
-      if (pv_issued > 0 && !(ok = warp_wait(&sm.bar_pvdone[X], (pv_issued - 1) & 1, abort_flag)))
-        break;
-      tc_fence_after();
-      if (__any_sync(0xffffffffu, raise) && pv_issued > 0) {
+    };
 #pragma unroll 1
-        for (int c = 0; c < 64; c += 16) {
-          float o[16];
-          tmem_ld16(tO + c, o);
+    for (int it = 0; it < nrow - (glob ? 1 : 0); ++it) {
+      const int j0 = (blo + it) * kHalf;
+      const int kind0 = chunk_kind(iw, j0, w, n), kind1 = chunk_kind(iw, j0 + 32, w, n);
+      wait_item();
+      if (!ok) break;
+      const uint32_t tS = tB + kHalf * buf;
+      float x[kHalf];
+      tmem_ld32(tS, x);
+      tmem_ld32(tS + 32, x + 32);
+      tmem_ld_wait();
+      if (kind0 == 1) mask_range(x, lo - j0, hi - j0);
+      if (kind1 == 1) mask_range(x + 32, lo - j0 - 32, hi - j0 - 32);
+      uint32_t pk[kHalf / 2];
+      float ls, os;
+      // at most twice: again with a raised reference for the rows whose sums
+      // came out too large under the old one (the maximum is looked for only
+      // then, and while a row of the warp has no reference yet; every row
+      // decides by its own values)
+      bool may = m_ref == -INFINITY;
+#pragma unroll 1
+      for (bool again = false;; again = true) {
+        if (__any_sync(0xffffffffu, may)) {
+          float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+          for (int ch = 0; ch < 2; ++ch)
+            if (ch ? kind1 : kind0)
+#pragma unroll
+              for (int k = 32 * ch; k < 32 * ch + 32; k += 8)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) mx[e] = fmax3(mx[e], x[k + 2 * e], x[k + 2 * e + 1]);
+          raise_to(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * kLogitScale2, may,
+                   it > 0);
+        }
+        const float nref = m_ref == -INFINITY ? 0.f : -m_ref;
+        const uint64_t n2 = f2_pack(nref, nref);
+        uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
+        float sq[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int ch = 0; ch < 2; ++ch) {
+          if (ch ? kind1 : kind0) {
+#pragma unroll
+            for (int k = 32 * ch; k < 32 * ch + 32; k += 2) {
+              float u, e;
+              f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, n2), u, e);
+              u = ex2(u);
+              e = ex2(e);
+              const uint32_t q = pack_bf16x2(u, e);
+              pk[k >> 1] = q;
+              if (k & 2) s2b = f2_add(s2b, f2_pack(u, e));
+              else s2a = f2_add(s2a, f2_pack(u, e));
+              const int c = (k >> 1) & 1;
+              sq[2 * c] = add_bf16_lo(sq[2 * c], q);
+              sq[2 * c + 1] = add_bf16_hi(sq[2 * c + 1], q);
+            }
+          } else {
+#pragma unroll
+            for (int k = 16 * ch; k < 16 * ch + 16; ++k) pk[k] = 0u;
+          }
+        }
+        float sa, sb, sc2, sd;
+        f2_unpack(s2a, sa, sb);
+        f2_unpack(s2b, sc2, sd);
+        ls = (sa + sb) + (sc2 + sd);
+        os = (sq[0] + sq[1]) + (sq[2] + sq[3]);
+        may = i < n && !(ls <= kMaxItemSum);
+        if (again || !__any_sync(0xffffffffu, may)) break;
+      }
+      lsum += ls;
+      osum += os;
+      tmem_st16(tS, pk);
+      tmem_st16(tS + 16, pk + 16);
+      tmem_st_wait();
+      hand_back();
+    }
+    // the global keys outside each row's band, and, with the row's LSE, the
+    // far-row column sums of the global keys (one partial per warp, merged
+    // later in a fixed order)
+    float lse = INFINITY;
+    if (glob) {
+      wait_item();
+      if (ok) {
+        // four global keys at a time; x = -inf where the band reaches the key
+        const uint32_t tS = tB + kHalf * buf;
+        auto load4 = [&](int g0, float* x) {
+          tmem_ld4(tS + g0, x);
           tmem_ld_wait();
 #pragma unroll
-          for (int k = 0; k < 16; ++k) o[k] *= f;
-          tmem_st16(tO + c, reinterpret_cast<const uint32_t*>(o));
-          tmem_st_wait();   // o is reused
+          for (int k = 0; k < 4; ++k)
+            x[k] = g0 + k < ng && abs(i - sm.gc[g0 + k]) > w ? x[k] * kLogitScale2 : -INFINITY;
+        };
+        float x[4], mx = -INFINITY;
+#pragma unroll 1
+        for (int g0 = 0; g0 < ng; g0 += 4) {
+          load4(g0, x);
+          mx = fmaxf(fmax3(mx, x[0], x[1]), fmaxf(x[2], x[3]));
         }
-      }
+        raise_to(mx, true, true);
+        const float nref = m_ref == -INFINITY ? 0.f : -m_ref;
+#pragma unroll 1
+        for (int g0 = 0; g0 < kMaxGlobal; g0 += 4) {
+          uint32_t pk[2] = {0u, 0u};
+          if (g0 < ng) {
+            load4(g0, x);
 #pragma unroll
-      for (int ch = 0; ch < 4; ++ch) tmem_st16(tP + 16 * ch, pk + 16 * ch);
-      tmem_st_wait();
-      tc_fence_before();
-      warp_arrive(&sm.bar_pready[X]);
-      ++pv_issued;
+            for (int k = 0; k < 4; k += 2) {
+              const float a = ex2(x[k] + nref), c = ex2(x[k + 1] + nref);
+              pk[k / 2] = pack_bf16x2(a, c);
+              lsum += a + c;
+              osum = add_bf16_hi(add_bf16_lo(osum, pk[k / 2]), pk[k / 2]);
+            }
+          }
+          tmem_st2(tS + kColPG + g0 / 2, pk);
+        }
+        if (valid) lse = m_ref + lg2(lsum);
+#pragma unroll 1
+        for (int g0 = 0; g0 < ng; g0 += 4) {
+          load4(g0, x);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) x[k] = valid ? ex2(x[k] - lse) : 0.f;
+          // two steps of a reduce-scatter, then plain sums: lane l holds key l >> 3
+#pragma unroll
+          for (int half = 2, bit = 16; half >= 1; half >>= 1, bit >>= 1)
+#pragma unroll
+            for (int k = 0; k < half; ++k) {
+              const bool upper = (lane & bit) != 0;
+              const float send = upper ? x[k] : x[k + half], mine = upper ? x[k + half] : x[k];
+              x[k] = mine + __shfl_xor_sync(0xffffffffu, send, bit);
+            }
+#pragma unroll
+          for (int o = 4; o > 0; o >>= 1) x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+          if ((lane & 7) == 0 && g0 + (lane >> 3) < ng)
+            p.gpart[(tile * 4 + warp) * kMaxGlobal + g0 + (lane >> 3)] = x[0];
+        }
+        tmem_st_wait();
+        hand_back();
+      }
+    } else if (valid) {
+      lse = m_ref + lg2(lsum);
     }
-
-    // ---- epilogue: LSE, the global keys and queries, the band's column
-    // sums, O
-    float lse = INFINITY;
-    const bool have_o = ok && pv_issued > 0 &&
-                        (ok = warp_wait(&sm.bar_pvdone[X], (pv_issued - 1) & 1, abort_flag));
-    if (have_o) lse = valid ? m_ref + lg2(lsum) : INFINITY;
-    if (active) sm.nlse[X][r] = -lse;
-
-    if (active && ngp) {
-      // Per-warp partial results (32 rows / 32 keys each), reduced with
-      // butterfly shuffles and merged later in a fixed order: no barrier here.
-      const size_t slot0 =
-          (((static_cast<size_t>(b) * p.H + h) * p.T + qt) * 4 + wq) * kMaxGlobal;
-      const int gme = lane >> 1;            // global index this lane reports
-      const bool writer = (lane & 1) == 0 && gme < ng;
-      float xg[kMaxGlobal], xt[kMaxGlobal];
-      const bool ok2 = ok && warp_wait(&sm.bar_sgend[X], 0, abort_flag);
-      if (ok2) {
-        tc_fence_after();
-        tmem_ld16(tS, xg);                  // S_G
-        tmem_ld16(tS + 16, xt);             // S_Gt
-        tmem_ld_wait();
-      }
-      // S_G and S_Gt are in registers: the S columns take the band pass while
-      // the global keys and queries are evaluated
-      tc_fence_before();
-      warp_arrive(&sm.bar_sfree[X]);
-      // far-row column sums of the global keys: rows outside the key's band
-      float e16[kMaxGlobal];
-#pragma unroll
-      for (int g = 0; g < kMaxGlobal; ++g) {
-        const bool use = ok2 && valid && g < ng && abs(i - sm.gc[g]) > p.w;
-        e16[g] = use ? ex2(fmaf(xg[g], kLogitScale2, -lse)) : 0.f;
-      }
-      const float gsum = warp_reduce16(e16, OpAdd());
-      if (writer) p.gpart[slot0 + gme] = gsum;
-      // (max, sum) of each global query over this warp's keys j = 128 qt + r
-      const bool key_ok = ok2 && (r0 + r < n);
-      float y[kMaxGlobal];
-#pragma unroll
-      for (int g = 0; g < kMaxGlobal; ++g) {
-        y[g] = (key_ok && g < ng) ? xt[g] * kLogitScale2 : -INFINITY;
-        e16[g] = y[g];
-      }
-      const float mme = warp_reduce16(e16, OpMax());
-#pragma unroll
-      for (int g = 0; g < kMaxGlobal; ++g) {
-        const float mg = __shfl_sync(0xffffffffu, mme, 2 * g);
-        e16[g] = mg == -INFINITY ? 0.f : ex2(y[g] - mg);
-      }
-      const float sme = warp_reduce16(e16, OpAdd());
-      if (writer) {
-        p.gstat[2 * (slot0 + gme)] = mme;
-        p.gstat[2 * (slot0 + gme) + 1] = sme;
-      }
-    }
+    const int last_pv = buf == 0 ? kBufs - 1 : buf - 1;   // P V of the row pass's last item
+    const uint32_t last_pv_use = buf == 0 ? use - 1 : use;
+    sm.nlse[r] = -lse;
+    named_sync_softmax();                 // every -LSE of the tile is in shared memory
 
     // Band pass (the column sums of Sec. "Extractor of Attention Scores"):
     // for each key j of the band, the sum over this tile's rows i of
     // exp2(S_ij scaled - LSE_i); global rows (LSE = +inf) and rows past the
     // end add nothing.  One thread per key column of S^T; written per query
-    // tile, summed over query tiles and heads in a fixed order by the
-    // finalisation.
-    if (active) named_sync_wg(X);   // every -LSE of the tile is in shared memory
-    const int nt = khiX - kloX + 1;
-    const uint64_t c2b = f2_pack(kLogitScale2, kLogitScale2);
-    for (int u = 0; ok && u < nt; ++u) {
-      const int j = (kloX + u) * kTile + r;   // key of this thread
-      if (!(ok = warp_wait(&sm.bar_sfull[X], (nt + u) & 1, abort_flag))) break;
-      tc_fence_after();
-      float x[128];
+    // tile, summed over query tiles and heads in a fixed order by the scores
+    // kernel.
+    float* const part = p.colpart + ((static_cast<size_t>(b) * p.H + h) * p.band_slots +
+                                     qt % p.band_slots) * p.L + r;
+    bool o_out = false;
+#pragma unroll 1
+    for (int u = 0; ok && u < nk; ++u) {
+      const int j0 = (klo + nk - 1 - u) * kTile, j = j0 + r, jw = j0 + 32 * warp;
+      uint64_t a2a = f2_pack(0.f, 0.f), a2b = a2a;
+#pragma unroll 1
+      for (int qh = 0; qh < 2; ++qh) {
+        if (!reaches(u, qh)) continue;
+        const int i0 = q0 + kHalf * qh;
+        // a warp's 32 keys against 32 queries: the relation is symmetric
+        const int kind0 = chunk_kind(jw, i0, w, n), kind1 = chunk_kind(jw, i0 + 32, w, n);
+        wait_item();
+        if (!ok) break;
+        const uint32_t tS = tB + kHalf * buf;
+        float x[kHalf];
+        tmem_ld32(tS, x);
+        tmem_ld32(tS + 32, x + 32);
+        tmem_ld_wait();
+        hand_back();
+        const float* lw = sm.nlse + kHalf * qh;
 #pragma unroll
-      for (int ch = 0; ch < 4; ++ch) tmem_ld32(tS + 32 * ch, x + 32 * ch);
-      tmem_ld_wait();
-      tc_fence_before();
-      warp_arrive(&sm.bar_sfree[X]);   // S^T is in registers
-      // query columns r0 + a .. r0 + e are in j's band (and in the sequence)
-      const int a = j - p.w - r0, e = min(j + p.w, n - 1) - r0;
-      if (!__all_sync(0xffffffffu, a <= 0 && e >= kTile - 1)) {
+        for (int ch = 0; ch < 2; ++ch) {
+          const int kind = ch ? kind1 : kind0;
+          if (kind == 0) continue;
+          // query columns of the chunk that are in j's band (and in the sequence)
+          if (kind == 1)
+            mask_range(x + 32 * ch, j - w - i0 - 32 * ch, min(j + w, n - 1) - i0 - 32 * ch);
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
-          const uint32_t keep = bit_range32(a - 32 * ch, e - 32 * ch);
-          if (__any_sync(0xffffffffu, keep != 0xffffffffu)) {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) {
-              const uint32_t out =
-                  ~static_cast<uint32_t>(static_cast<int32_t>(keep << (31 - k)) >> 31);
-              x[32 * ch + k] =
-                  __uint_as_float((__float_as_uint(x[32 * ch + k]) & ~out) | (0xff800000u & out));
-            }
+          for (int k = 32 * ch; k < 32 * ch + 32; k += 4) {
+            const float4 l4 = *reinterpret_cast<const float4*>(lw + k);
+            float e0, e1, e2, e3;
+            f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, f2_pack(l4.x, l4.y)), e0, e1);
+            f2_unpack(f2_fma(f2_pack(x[k + 2], x[k + 3]), c2, f2_pack(l4.z, l4.w)), e2, e3);
+            a2a = f2_add(a2a, f2_pack(ex2(e0), ex2(e1)));
+            a2b = f2_add(a2b, f2_pack(ex2(e2), ex2(e3)));
           }
         }
       }
-      const float* lw = sm.nlse[X];
-      uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
-#pragma unroll
-      for (int k = 0; k < kTile; k += 4) {
-        const float4 l4 = *reinterpret_cast<const float4*>(lw + k);
-        float e0, e1, e2, e3;
-        f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2b, f2_pack(l4.x, l4.y)), e0, e1);
-        f2_unpack(f2_fma(f2_pack(x[k + 2], x[k + 3]), c2b, f2_pack(l4.z, l4.w)), e2, e3);
-        s2a = f2_add(s2a, f2_pack(ex2(e0), ex2(e1)));
-        s2b = f2_add(s2b, f2_pack(ex2(e2), ex2(e3)));
-      }
       float sa, sb, sc2, sd;
-      f2_unpack(s2a, sa, sb);
-      f2_unpack(s2b, sc2, sd);
-      if (j < n)
-        p.colpart[((static_cast<size_t>(b) * p.H + h) * p.L + j) * band_slots + qt % band_slots] =
-            (sa + sc2) + (sb + sd);
-    }
-
-    // ---- O: its rows leave through this warp's quarter of its Q tile; every
-    // MMA that read the tile completed before the last S^T was awaited
-    if (ok && have_o && v.O != nullptr) {
-      tc_fence_after();
-      const float inv = 1.f / osum;
-      uint8_t* stage = Qs + X * kTileBytes + wq * 4096;
-#pragma unroll
-      for (int c = 0; c < 64; c += 32) {
-        float o[32];
-        tmem_ld32(tO + c, o);
-        tmem_ld_wait();
-#pragma unroll
-        for (int k = 0; k < 32; k += 8)
-          stage_row_piece<8>(stage, (c + k) >> 3,
-                          make_uint4(pack_bf16x2(o[k] * inv, o[k + 1] * inv),
-                                     pack_bf16x2(o[k + 2] * inv, o[k + 3] * inv),
-                                     pack_bf16x2(o[k + 4] * inv, o[k + 5] * inv),
-                                     pack_bf16x2(o[k + 6] * inv, o[k + 7] * inv)));
+      f2_unpack(a2a, sa, sb);
+      f2_unpack(a2b, sc2, sd);
+      if (ok && j < n) part[j0] = (sa + sc2) + (sb + sd);
+      if (!o_out) {
+        // ---- O: its rows leave through the last tile's V slot
+        o_out = true;
+        ok = ok && warp_wait_poll(&sm.bar_pv[last_pv], last_pv_use & 1, abort_flag);
+        tc_fence_after();
+        if (ok && v.O != nullptr) {
+          const float inv = 1.f / osum;
+          uint8_t* stage = Slots + vd_slot * kTileBytes + warp * 4096;
+#pragma unroll 1
+          for (int c = 0; c < 64; c += 8) {
+            float o[8];
+            tmem_ld8(tO + c, o);
+            tmem_ld_wait();
+            stage_row_piece<8>(stage, c >> 3,
+                               make_uint4(pack_bf16x2(o[0] * inv, o[1] * inv),
+                                          pack_bf16x2(o[2] * inv, o[3] * inv),
+                                          pack_bf16x2(o[4] * inv, o[5] * inv),
+                                          pack_bf16x2(o[6] * inv, o[7] * inv)));
+          }
+          __syncwarp();
+          // four rows an instruction, eight lanes a row
+          const uint32_t rows = __ballot_sync(0xffffffffu, valid) >> (lane >> 3);
+          uint16_t* dst = v.O + ((static_cast<size_t>(b) * p.L + iw + (lane >> 3)) * p.H + h) *
+                                    kHeadDim + 8 * (lane & 7);
+#pragma unroll 2
+          for (int k = 0; k < 32; k += 4, dst += static_cast<size_t>(4) * p.H * kHeadDim) {
+            const uint4 val = *reinterpret_cast<const uint4*>(
+                stage + stage_offset<8>(k + (lane >> 3), lane & 7));
+            if ((rows >> k) & 1u) *reinterpret_cast<uint4*>(dst) = val;
+          }
+        }
+        fence_proxy_async_smem();         // ... before the copy of V into it
+        tc_fence_before();
+        warp_arrive(&sm.bar_stage);
       }
-      flush_staged_rows<8>(stage,
-                        v.O + ((static_cast<size_t>(b) * p.L + r0 + 32 * wq) * p.H + h) * kHeadDim,
-                        static_cast<size_t>(p.H) * kHeadDim, __ballot_sync(0xffffffffu, valid));
+      if (glob && u == u_d) {             // S_Gt of the tile's keys, for warps 6 and 7
+        wait_item();
+        if (!ok) break;
+        const uint32_t tS = tB + kHalf * buf;
+#pragma unroll 1
+        for (int g0 = 0; g0 < ng; g0 += 4) {
+          float y[4];
+          tmem_ld4(tS + g0, y);
+          tmem_ld_wait();
+#pragma unroll
+          for (int k = 0; k < 4; ++k)   // key i
+            gx[(g0 + k) * kTile + r] = i < n ? y[k] * kLogitScale2 : -INFINITY;
+        }
+        hand_back();
+        tc_fence_before();
+        warp_arrive(&sm.bar_gx);
+      }
     }
   }
 
   tc_fence_before();
-  __threadfence();   // O, the partial sums and statistics of this CTA ...
   __syncthreads();
-  if (warp == 9) {
+  if (warp == 4) {
     tc_fence_after();
-    tmem_dealloc(tm, 512);
+    tmem_dealloc(tm, 256);
   }
   if (tid == 0) {
     if (sm.abort) atomicOr(p.status, kStatusTimeout);
-    red_release_add_u32(p.rows_done + b * p.H + h, 1u);   // ... are visible to the cols CTAs
+    // O, the partial sums and statistics of this CTA (ordered before this by
+    // the barrier) are visible to the scores CTAs that see the count
+    red_release_add_u32(p.rows_done + b * p.H, 1u);
   }
 }
 
@@ -659,24 +843,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1)
 // Tensor memory (256 columns, so that two CTAs share an SM) per warpgroup X:
 // S^T against the global queries [16 X, +16), the global rows' P V
 // [64 + 64 X, +64).
-// The band rows' column sums of key j from the rows kernel, one per query tile
-// qlo..qhi in tile order (slot = tile mod kSlots); entries past qhi are 0.
-template <int kSlots>
-__device__ __forceinline__ void load_band_parts(float (&part)[kWideBandTiles], const LayerParams& p,
-                                                int b, int h, int j, int qlo, int qhi, bool use) {
-  const float* cp = p.colpart + ((static_cast<size_t>(b) * p.H + h) * p.L + j) * kSlots;
-#pragma unroll
-  for (int u = 0; u < kWideBandTiles; ++u)
-    part[u] = (u < kSlots && use && qlo + u <= qhi) ? __ldcg(cp + (qlo + u) % kSlots) : 0.f;
-}
-
 constexpr int kColsThreads = 320;
-// The global rows' P is the A operand of an M = 128 MMA whose rows past the 16
-// global rows are never used: each 64-key block of that A tile holds its 16
-// valid rows (2 KB) and lets the MMA read the following rows from whatever
-// shared memory comes next (the K and V tiles), so only 2 KB is reserved.
-constexpr uint32_t kPgBlock = 2 * 1024;
-
 struct ColsSmem {
   uint64_t bar_kv;
   uint64_t bar_sfull[2], bar_sfree[2], bar_sg[2], bar_pg[2], bar_og[2], bar_fin;
@@ -685,16 +852,10 @@ struct ColsSmem {
   int gc[kMaxGlobal];
   float lse_g[kMaxGlobal];
   int flag, flag2;
-  int gnew[kMaxGlobal];
+  FinalSmem<kColsThreads> fin;
   // each key tile's part of the global rows' P V (warpgroup X), added in
   // tile order into the pair's part
   alignas(16) float ogx[2][kMaxGlobal][kHeadDim];   // read and written as float4
-  // sequence compaction: per (round, warp) ballot of kept tokens and the
-  // exclusive prefix of their counts
-  uint32_t kbits[(kMaxLen + kColsThreads - 1) / kColsThreads][kColsThreads / 32];
-  int kpre[(kMaxLen + kColsThreads - 1) / kColsThreads][kColsThreads / 32];
-  int last_pos;
-  int total;
 };
 
 // dynamic shared memory: the global rows' P blocks (2 per warpgroup), K and V
@@ -702,9 +863,6 @@ struct ColsSmem {
 constexpr uint32_t kColsDyn = 4 * kPgBlock + kTileBytes * 4 + kGTileBytes + 1024;
 static_assert(3 * kPgBlock + kTileBytes <= 4 * kPgBlock + 4 * kTileBytes,
               "the A operand's unused rows stay inside the shared memory");
-
-__device__ void finalize_sequence(const LayerParams& p, const LayerView& v, int b, int n,
-                                  ColsSmem& sm, uint8_t* scratch);
 
 __global__ void __launch_bounds__(kColsThreads, 2)
     sc_cols_kernel(const __grid_constant__ TensorMaps maps, const __grid_constant__ LayerParams p) {
@@ -830,17 +988,17 @@ __global__ void __launch_bounds__(kColsThreads, 2)
     // sums, statistics and the cleared global-row outputs are read below)
     if (tid == 0)
       wait_count(p.rows_done + b * p.H + h,
-                 static_cast<uint32_t>((p.wide || p.band) ? Tn : Tp), abort_flag);
+                 static_cast<uint32_t>(Tn), abort_flag);
     asm volatile("bar.sync 3, 256;" ::: "memory");
     // every load of the prologue is issued before any is used: this key's
     // band-row column sums of the query tiles of its band (one per tile, from
     // the rows kernel) and, per warp, the (max, sum) pieces of global rows
     // warp and warp + 8
-    float part[kWideBandTiles];
-    if (p.band_slots == kMaxBandTiles)
-      load_band_parts<kMaxBandTiles>(part, p, b, h, j, qloX, qhiX, active && j < n);
-    else
-      load_band_parts<kWideBandTiles>(part, p, b, h, j, qloX, qhiX, active && j < n);
+    float part[kMaxBandTiles];   // (slot = query tile mod kMaxBandTiles)
+    const float* cp = p.colpart + ((static_cast<size_t>(b) * p.H + h) * p.L + j) * kMaxBandTiles;
+#pragma unroll
+    for (int u = 0; u < kMaxBandTiles; ++u)
+      part[u] = (active && j < n && qloX + u <= qhiX) ? __ldcg(cp + (qloX + u) % kMaxBandTiles) : 0.f;
     // lane k takes entries k, k+32, k+64, k+96 of the 4 Tn (key tile, warp
     // slice) pieces; the warp combines them in a fixed order
     const size_t base_slot = (static_cast<size_t>(b) * p.H + h) * p.T * 4 * kMaxGlobal;
@@ -896,7 +1054,7 @@ __global__ void __launch_bounds__(kColsThreads, 2)
     // band rows: the query tiles' sums in tile order
     float acc = 0.f;
 #pragma unroll
-    for (int u = 0; u < kWideBandTiles; ++u) acc += part[u];
+    for (int u = 0; u < kMaxBandTiles; ++u) acc += part[u];
     // far rows of the global keys among this warp's keys (gc increases with
     // g, so they are consecutive entries of the list)
     if (far_g >= 0) {
@@ -1076,122 +1234,7 @@ __global__ void __launch_bounds__(kColsThreads, 2)
   __syncthreads();
   if (!sm.flag) return;
   __threadfence();
-  finalize_sequence(p, v, b, n, sm, base);
-}
-
-struct BlockSync {
-  __device__ __forceinline__ void operator()() const { __syncthreads(); }
-};
-
-// Order-preserving compaction of sequence b's kept tokens, the next layer's
-// global list, and the bf16 outputs of the global rows.  One CTA; token c is
-// handled by thread c % kColsThreads in round c / kColsThreads (coalesced
-// loads, all issued at once); output slots come from warp ballots and a
-// fixed-order prefix over (round, warp).  Under the top-ratio rule the keep
-// flags come from the cut over all n scores, found here (`scratch`: shared
-// memory the CTA no longer uses, for the selection's histogram and tie flags).
-__device__ void finalize_sequence(const LayerParams& p, const LayerView& v, int b, int n,
-                                  ColsSmem& sm, uint8_t* scratch) {
-  constexpr int kRounds = (kMaxLen + kColsThreads - 1) / kColsThreads;
-  constexpr int kWarps = kColsThreads / 32;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint8_t* keep = p.keep + static_cast<size_t>(b) * p.L;
-  const int32_t* pos = v.pos + static_cast<size_t>(b) * p.L;
-  int32_t* pos_out = v.pos_out + static_cast<size_t>(b) * p.L;
-  bool kf[kRounds];
-  int32_t ps[kRounds];
-  if (p.keep_rule == kKeepTopRatio) {
-    const float* sc = v.scores + static_cast<size_t>(b) * p.L;
-    uint32_t key[kRounds];
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-      const int c = r * kColsThreads + tid;
-      key[r] = (c >= 1 && c < n) ? select_key(__ldcg(sc + c)) : 0u;
-      ps[r] = c < n ? __ldcg(pos + c) : 0;
-    }
-    SelectSmem& ss = *reinterpret_cast<SelectSmem*>(scratch);
-    uint8_t* tie = scratch + sizeof(SelectSmem);
-    uint32_t cut;
-    int ties, eq;
-    radix_cut<kColsThreads, kRounds>(key, top_count(v.alpha, n) - 1, n - 1, ss, tid, BlockSync(),
-                                     cut, ties, eq);
-    const bool split = eq > ties;   // an exact tie straddles the cut
-    if (split) rank_ties<kColsThreads, kRounds>(key, cut, ties, n, tie, tid, BlockSync());
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-      const int c = r * kColsThreads + tid;
-      kf[r] = c < n && (c == 0 || key[r] > cut || (key[r] == cut && (!split || tie[c] == 2)));
-    }
-  } else {
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-      const int c = r * kColsThreads + tid;
-      kf[r] = c < n && __ldcg(keep + c) != 0;
-      ps[r] = c < n ? __ldcg(pos + c) : 0;
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    const uint32_t bits = __ballot_sync(0xffffffffu, kf[r]);
-    if (lane == 0) sm.kbits[r][warp] = bits;
-  }
-  if (tid < kMaxGlobal) sm.gnew[tid] = -1;
-  __syncthreads();
-  if (warp == 0) {
-    // prefix over (round, warp) in order: lane l covers entries l, l+32, ...
-    constexpr int kEntries = kRounds * kWarps;
-    int cnt[(kEntries + 31) / 32];
-    int run = 0;
-#pragma unroll
-    for (int u = 0; u < (kEntries + 31) / 32; ++u) {
-      const int e = u * 32 + lane;
-      cnt[u] = e < kEntries ? __popc(sm.kbits[e / kWarps][e % kWarps]) : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < (kEntries + 31) / 32; ++u) {
-      int x = cnt[u];
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, off);
-        if (lane >= off) x += y;
-      }
-      const int e = u * 32 + lane;
-      if (e < kEntries) sm.kpre[e / kWarps][e % kWarps] = run + x - cnt[u];
-      run += __shfl_sync(0xffffffffu, x, 31);
-    }
-    if (lane == 0) sm.total = run;
-  }
-  __syncthreads();
-  const uint32_t below = (1u << lane) - 1u;
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    if (!kf[r]) continue;
-    const int out = sm.kpre[r][warp] + __popc(sm.kbits[r][warp] & below);
-    pos_out[out] = ps[r];
-    if (p.kept_cur) p.kept_cur[static_cast<size_t>(b) * p.L + out] = r * kColsThreads + tid;
-    if (out == sm.total - 1) sm.last_pos = ps[r];
-  }
-  // next-layer index of each surviving global token
-  const int ng = min(__ldcg(v.ng + b), kMaxGlobal);
-  if (tid < ng) {
-    const int c = sm.gc[tid], r = c / kColsThreads, t = c % kColsThreads;
-    const uint32_t bits = sm.kbits[r][t >> 5];
-    if ((bits >> (t & 31)) & 1u) sm.gnew[tid] = sm.kpre[r][t >> 5] + __popc(bits & ((1u << (t & 31)) - 1u));
-  }
-  __syncthreads();
-  if (tid == 0) {
-    const int total = sm.total;
-    int m = 0;
-    for (int g = 0; g < ng; ++g)
-      if (sm.gnew[g] >= 0) v.gcur_out[b * kMaxGlobal + m++] = sm.gnew[g];
-    v.ng_out[b] = m;
-    v.len_out[b] = total;
-    if (p.tail_from != nullptr && total <= p.tail_max) p.tail_from[b] = v.layer + 1;
-    // the survivors are original positions 0..total-1 exactly when the last one is total-1
-    v.ident_out[b] = (!p.no_ident && (total == 0 || sm.last_pos == total - 1)) ? 1 : 0;
-    p.cnt_seq[b] = 0u;
-    for (int hh = 0; hh < p.H; ++hh) p.rows_done[b * p.H + hh] = 0u;
-  }
+  finalize_sequence<kColsThreads>(p, v, b, n, sm.fin, sm.gc, base);
 }
 
 // ---------------------------------------------------------------------------
@@ -1502,19 +1545,12 @@ cudaError_t configure_band();
 cudaError_t configure_kernels() {
   // the attention kernels use most of an SM's shared memory
   cudaError_t e = configure_band();
-  for (auto k : {sc_rows_kernel<false>, sc_rows_kernel<true>}) {
-    // the warpgroups' register split (setmaxnreg) needs the whole launch
-    // allocation: with fewer registers a thread, an increase would never be granted
-    cudaFuncAttributes fa;
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
-    if (e == cudaSuccess && fa.numRegs < kRowsLaunchRegs) e = cudaErrorInvalidConfiguration;
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(kRowsDyn));
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                               cudaSharedmemCarveoutMaxShared);
-  }
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(sc_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(kRowsDyn));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(sc_rows_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(sc_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kColsDyn));
@@ -1528,14 +1564,14 @@ cudaError_t launch_band(const TensorMaps& m, const LayerParams& p, int sms, cuda
 
 cudaError_t launch_rows(const TensorMaps& m, const LayerParams& p, cudaStream_t st) {
   if (p.band) return launch_band(m, p, p.sms, st);
-  if (p.wide)
-    return launch_chained(sc_rows_kernel<true>, dim3(p.B * p.H * p.T), dim3(kRowsThreads),
-                          kRowsDyn, st, m, p);
-  return launch_chained(sc_rows_kernel<false>, dim3(p.B * p.H * ((p.T + 1) / 2)),
-                        dim3(kRowsThreads), kRowsDyn, st, m, p);
+  return launch_chained(sc_rows_kernel, dim3(p.B * p.H * p.T), dim3(kRowsThreads), kRowsDyn, st, m,
+                        p);
 }
 
+cudaError_t launch_scores(const LayerParams& p, cudaStream_t st);
+
 cudaError_t launch_cols(const TensorMaps& m, const LayerParams& p, cudaStream_t st) {
+  if (!p.band) return launch_scores(p, st);
   dim3 grid(p.B * p.H * ((p.T + 1) / 2));
   return launch_chained(sc_cols_kernel, grid, dim3(kColsThreads), kColsDyn, st, m, p);
 }

@@ -50,6 +50,12 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
 }
 
+// The same, polling without a suspend-time hint.
+__device__ __forceinline__ bool warp_wait_poll(uint64_t* bar, uint32_t parity,
+                                               volatile int* abort) {
+  return __all_sync(0xffffffffu, mbar_wait_poll(bar, parity, abort));
+}
+
 // The per-layer fields of this launch: as given, or (device-driven layer
 // loop) the layer-0 values advanced to layer *dev_layer.
 __device__ __forceinline__ LayerView layer_view(const LayerParams& p) {
