@@ -46,6 +46,7 @@ constexpr int kTailTiles = (kTailMax + kTile - 1) / kTile;   // 128-row tiles (3
 constexpr uint32_t kTailOpBytes = kTailTiles * kTileBytes;   // rows of one tensor (48 KB)
 constexpr int kTailChunks = kTailMax / 32;                    // 32-token chunks (12)
 static_assert(kTailMax <= 384, "a second key half must fit beside O in tensor memory");
+constexpr float kMaxChunkSum = 16777216.f;                   // 2^24 (see half_softmax)
 constexpr uint32_t kTailStageBytes = 8 * 2048;                // O row staging, 2 KB per softmax warp
 // column sums of every head, [layer parity][head][column], written by the
 // CTA of that head into every CTA of the cluster
@@ -87,7 +88,7 @@ struct TailSync {   // the 256 softmax threads
 };
 
 __device__ __forceinline__ bool tail_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
+  return __all_sync(0xffffffffu, mbar_wait_poll(bar, parity, abort));
 }
 
 // Bits a..b (inclusive, clipped to 0..31) of a 32-bit word.
@@ -223,6 +224,7 @@ __global__ void __launch_bounds__(kTailThreads, 1)
       // same piece of Q, K and V from one address computation
       const size_t tok0 = (static_cast<size_t>(l) * B + b) * L;
       const int piece = tid & 7;
+#pragma unroll 2
       for (int r = tid >> 3; r < n; r += kTailThreads / 8) {
         const size_t off = ((tok0 + sm.pos[cur][r]) * H + h) * kHeadDim + 8 * piece;
         const uint32_t so = sw128_offset(r, piece);
@@ -233,6 +235,7 @@ __global__ void __launch_bounds__(kTailThreads, 1)
       if (l + 1 < n_layers && !p.src_host) {
         // the next layer's tokens are a subset of the current ones
         const size_t tok1 = (static_cast<size_t>(l + 1) * B + b) * L;
+#pragma unroll 1
         for (int r = tid; r < n; r += kTailThreads) {
           const size_t off = ((tok1 + sm.pos[cur][r]) * H + h) * kHeadDim;
 #pragma unroll
@@ -247,12 +250,37 @@ __global__ void __launch_bounds__(kTailThreads, 1)
     __syncthreads();
     tc_fence_after();
 
+    // O of the warp's 32 rows, bf16 pairs, until it is stored: through the staging
+    // area in two column halves of 64 bytes (no O but the last layer's when O is
+    // not kept)
+    uint32_t opk[32];
+    bool o_held = false;
+    int o_row = 0;
+    uint32_t o_rows = 0u;
+    auto store_o = [&]() {
+      uint16_t* const Ol = out_O != nullptr ? out_O + static_cast<size_t>(l) * B * L * H * kHeadDim
+                           : l == n_layers - 1 ? out_O_last : nullptr;
+      if (Ol == nullptr) return;
+      uint8_t* stage = base + 3 * kTailOpBytes + warp * 2048;
+      uint16_t* row0 = Ol + ((static_cast<size_t>(b) * L + o_row) * H + h) * kHeadDim;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          stage_row_piece<4>(stage, k, make_uint4(opk[16 * c + 4 * k], opk[16 * c + 4 * k + 1],
+                                                  opk[16 * c + 4 * k + 2], opk[16 * c + 4 * k + 3]));
+        flush_staged_rows<4>(stage, row0 + 32 * c, static_cast<size_t>(H) * kHeadDim, o_rows);
+      }
+    };
+
     if (warp >= 8) {
       // ------------------------------------------------------- MMA issue
       const int X = warp - 8;
       if (lane == 0 && X < nq && *abort_flag == 0) {
         const uint32_t tR = tm + 256u * X;              // this warpgroup's columns
-        const uint32_t id_pv = idesc_bf16(128, 64, false, true);
+        const uint32_t q_d = sdesc_lo(q_a), k_d = sdesc_lo(k_a), v_d = sdesc_lo(v_a);
+        constexpr uint32_t kTileD = kTileBytes >> 4;    // in descriptors
+        constexpr uint32_t id_pv = idesc_bf16(128, 64, false, true);
         bool first = true, ok = true;
         // the warpgroup's columns may be overwritten: the previous contents are read
         auto region = [&]() -> bool {
@@ -260,68 +288,45 @@ __global__ void __launch_bounds__(kTailThreads, 1)
             first = false;
             return true;
           }
-          return mbar_wait(&sm.bar_sfree[X], (n_sfree++) & 1, abort_flag);
+          return mbar_wait_poll(&sm.bar_sfree[X], (n_sfree++) & 1, abort_flag);
         };
-        auto ready = [&]() -> bool {
-          return mbar_wait(&sm.bar_pready[X], (n_ready++) & 1, abort_flag);
-        };
-        auto issue_s = [&](int qt, int kh) {   // S of query tile qt against key half kh
-          const int N = round16(min(256, n - 256 * kh));
-          const uint32_t id = idesc_bf16(128, N, false, false);
+        // D[128 x N] = A[128 x 64] B[N x 64]^T over the rows (columns) of half kh
+        auto issue_qk = [&](uint32_t dst, uint32_t a_d, uint32_t b_d, int kh, uint64_t* bar) {
+          const uint32_t id = idesc_bf16(128, 0, false, false) |
+                              (static_cast<uint32_t>(round16(min(256, n - 256 * kh)) >> 3) << 17);
+          b_d += kh * 2 * kTileD;
           tc_fence_after();
 #pragma unroll
           for (int k = 0; k < kHeadDim / 16; ++k)
-            umma_bf16(tR, sdesc_sw128(q_a + qt * kTileBytes + 32 * k),
-                      sdesc_sw128(k_a + kh * 2 * kTileBytes + 32 * k), id, k > 0);
-          umma_commit(&sm.bar_sfull[X]);
+            umma_bf16_lo(dst, a_d + 2 * k, b_d + 2 * k, id, k > 0);
+          umma_commit(bar);
         };
-        auto issue_pv = [&](int kh, bool acc) {   // O (+)= P V over key half kh
-          const int N = round16(min(256, n - 256 * kh));
-          tc_fence_after();
-          for (int k = 0; k < N / 16; ++k)
-            umma_bf16_ts(tR + 128u, tR + 8u * k, sdesc_sw128(v_a + kh * 2 * kTileBytes + 2048u * k),
-                         id_pv, (acc || k > 0) ? 1u : 0u);
-          umma_commit(&sm.bar_odone[X]);
-        };
-        auto issue_st = [&](int kt, int qh, uint32_t dst) {   // S^T of key tile kt, query half qh
-          const int N = round16(min(256, n - 256 * qh));
-          const uint32_t id = idesc_bf16(128, N, false, false);
-          tc_fence_after();
-#pragma unroll
-          for (int k = 0; k < kHeadDim / 16; ++k)
-            umma_bf16(dst, sdesc_sw128(k_a + kt * kTileBytes + 32 * k),
-                      sdesc_sw128(q_a + qh * 2 * kTileBytes + 32 * k), id, k > 0);
-          umma_commit(&sm.bar_stfull[X]);
-        };
-        for (int r = 0; ok && r < 2; ++r) {
-          const int qt = X + 2 * r;
-          if (qt >= nq) break;
-          if (nkh == 1) {
-            if (!(ok = region())) break;
-            issue_s(qt, 0);
-            // one query tile: the other half of tensor memory takes S^T at once
-            if (nq == 1) issue_st(0, 0, tm + 256u);
-            if (!(ok = ready())) break;
-            issue_pv(0, false);
-          } else {
-            if (!(ok = region())) break;
-            issue_s(qt, 0);
-            if (!(ok = ready())) break;
-            issue_pv(0, false);
-            // key half 1 has at most 128 columns: its S lands on P of half 0
-            // (not on O) after that half's P V in issue order, so it may be
-            // issued at once
-            issue_s(qt, 1);
-            if (!(ok = ready())) break;
-            issue_pv(1, true);
-          }
-        }
-        for (int r = 0; ok && nq > 1 && r < 2; ++r) {
-          const int kt = X + 2 * r;
-          if (kt >= nq) break;
-          for (int qh = 0; ok && qh < nkh; ++qh) {
-            if (!(ok = region())) break;
-            issue_st(kt, qh, tR);
+        // rows: per query tile, S of each key half and O (+)= P V over it; half 1
+        // has at most 128 columns: its S lands on P of half 0 (not on O) after
+        // that half's P V in issue order.  Then, per key tile, S^T of each query
+        // half (with one tile in all the other half of tensor memory takes it at
+        // once).
+#pragma unroll 1
+        for (int r = 0; ok && r < 4; ++r) {
+          const int t = X + 2 * (r & 1);
+          if (t >= nq) continue;
+          const bool rows = r < 2;
+          if (!rows && nq == 1) break;
+#pragma unroll 1
+          for (int kh = 0; ok && kh < nkh; ++kh) {
+            if ((kh == 0 || !rows) && !(ok = region())) break;
+            issue_qk(tR, (rows ? q_d : k_d) + t * kTileD, rows ? k_d : q_d, kh,
+                     rows ? &sm.bar_sfull[X] : &sm.bar_stfull[X]);
+            if (!rows) continue;
+            if (nq == 1) issue_qk(tm + 256u, k_d, q_d, 0, &sm.bar_stfull[X]);
+            if (!(ok = mbar_wait_poll(&sm.bar_pready[X], (n_ready++) & 1, abort_flag))) break;
+            tc_fence_after();
+            const int steps = round16(min(256, n - 256 * kh)) / 16;
+#pragma unroll 2
+            for (int k = 0; k < steps; ++k)
+              umma_bf16_ts_lo(tR + 128u, tR + 8u * k, v_d + kh * 2 * kTileD + 128 * k, id_pv,
+                              (kh > 0 || k > 0) ? 1u : 0u);
+            umma_commit(&sm.bar_odone[X]);
           }
         }
         if (ok) region();   // the last release of the layer
@@ -341,71 +346,115 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         me.all = w >= n - 1 || ((sm.gbits[cur][i >> 5] >> (i & 31)) & 1u);
         return me;
       };
-      // row maximum over the keys of half kh (S in tensor memory)
-      auto half_max = [&](const Partners& me, int kh, float mx) {
-        const int nh = min(256, n - 256 * kh);
-        for (int q2 = 0; q2 < (nh + 63) >> 6; ++q2) {
-          float x[64];
-          tmem_ld32(tR + 64 * q2, x);
-          tmem_ld32(tR + 64 * q2 + 32, x + 32);
-          tmem_ld_wait();
+      // Softmax of half kh (S in tensor memory) against the row's reference, 32
+      // keys at a time: P = exp2(S - ref), written as bf16 pairs over the first
+      // half of the columns (each chunk's pairs land on columns that this or an
+      // earlier chunk has read).  The reference is the maximum of the first chunk
+      // that the row attends to; a chunk whose exponentials sum to more than
+      // kMaxChunkSum raises it by a whole power of two, by which everything
+      // formed so far (the half's P, the sums, and O of the half before) is
+      // scaled exactly.
+      // lsum: the sum of the exponentials (fp32: the row's LSE, which the column
+      // sums use); osum: the sum of the same values rounded to the bf16 that P V
+      // multiplies (the normaliser of O, so that O is a weighted mean of V rows
+      // whatever the rounding of P).
+      // The chunk loop stays rolled: the layer's code runs once per layer and has
+      // to stay in the instruction caches.
+      auto half_softmax = [&](const Partners& me, int kh, float& ref, float& lsum, float& osum) {
+        const int chunks = (round16(min(256, n - 256 * kh)) + 31) >> 5;
+#pragma unroll 1
+        for (int q = 0; q < chunks; ++q) {
+          const uint32_t in = partner_mask(me, sm, cur, 8 * kh + q, n);
+          uint32_t pk[16];
+          if (!__any_sync(0xffffffffu, in != 0u)) {   // outside every row's window
 #pragma unroll
-          for (int hq = 0; hq < 2; ++hq) {
-            apply_mask(x + 32 * hq, partner_mask(me, sm, cur, 8 * kh + 2 * q2 + hq, n));
+            for (int k = 0; k < 16; ++k) pk[k] = 0u;
+          } else {
+            float x[32];
+            tmem_ld32(tR + 32 * q, x);
+            tmem_ld_wait();
+            apply_mask(x, in);
+            float ls, os;
+            bool may = in != 0u && ref == -INFINITY;
+#pragma unroll 1
+            for (bool again = false;; again = true) {   // again: under a raised reference
+              if (__any_sync(0xffffffffu, may)) {
+                float mx = -INFINITY;
 #pragma unroll
-            for (int k = 0; k < 32; k += 2) mx = fmax3(mx, x[32 * hq + k], x[32 * hq + k + 1]);
-          }
-        }
-        return mx;
-      };
-      // P = exp2(S - max) over half kh, written as bf16 pairs over the first
-      // half of its columns (each step's pairs land on columns this or an
-      // earlier step has read); returns the half's row sum
-      // Returns the half's sum of the exponentials (fp32: the row's LSE, which
-      // the column sums use) and adds to *osum the same values rounded to the
-      // bf16 that P V multiplies (the normaliser of O, so that O is a weighted
-      // mean of V rows whatever the rounding of P).
-      auto half_exp = [&](const Partners& me, int kh, float nmc, float* osum) {
-        const int nh = min(256, n - 256 * kh);
-        const uint64_t n2 = f2_pack(nmc, nmc);
-        uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
-        float la = 0.f, lb = 0.f, lc = 0.f, ld = 0.f;
-        for (int q2 = 0; q2 < (nh + 63) >> 6; ++q2) {
-          float x[64];
-          tmem_ld32(tR + 64 * q2, x);
-          tmem_ld32(tR + 64 * q2 + 32, x + 32);
-          tmem_ld_wait();
+                for (int k = 0; k < 32; k += 2) mx = fmax3(mx, x[k], x[k + 1]);
+                mx *= kLogitScale2;
+                float f = 1.f;
+                if (may && mx > ref + 8.f) {
+                  if (ref == -INFINITY) {   // all sums and P so far are 0
+                    ref = mx;
+                  } else {
+                    const float up = ceilf(mx - ref);
+                    f = ex2(-up);
+                    ref += up;
+                    lsum *= f;
+                    osum *= f;
+                  }
+                }
+                if (__any_sync(0xffffffffu, f != 1.f)) {
+#pragma unroll 1
+                  for (int c = 0; c < 16 * q; c += 8) {
+                    float w8[8];
+                    tmem_ld8(tR + c, w8);
+                    tmem_ld_wait();
+                    uint32_t u[8];
 #pragma unroll
-          for (int hq = 0; hq < 2; ++hq) {
-            float* xh = x + 32 * hq;
-            apply_mask(xh, partner_mask(me, sm, cur, 8 * kh + 2 * q2 + hq, n));
-            uint32_t pk[16];
+                    for (int k = 0; k < 8; ++k) {
+                      const uint32_t b2 = __float_as_uint(w8[k]);
+                      u[k] = pack_bf16x2(__uint_as_float(b2 << 16) * f,
+                                         __uint_as_float(b2 & 0xffff0000u) * f);
+                    }
+                    tmem_st8(tR + c, u);
+                    tmem_st_wait();
+                  }
+#pragma unroll 1
+                  for (int c = 0; kh > 0 && c < 64; c += 8) {
+                    float o[8];
+                    tmem_ld8(tO + c, o);
+                    tmem_ld_wait();
 #pragma unroll
-            for (int k = 0; k < 32; k += 2) {
-              float u, v;
-              f2_unpack(f2_fma(f2_pack(xh[k], xh[k + 1]), c2, n2), u, v);
-              u = ex2(u);
-              v = ex2(v);
-              if (k & 2) s2b = f2_add(s2b, f2_pack(u, v));
-              else s2a = f2_add(s2a, f2_pack(u, v));
-              pk[k >> 1] = pack_bf16x2(u, v);
-              if (k & 2) {
-                lc = add_bf16_lo(lc, pk[k >> 1]);
-                ld = add_bf16_hi(ld, pk[k >> 1]);
-              } else {
-                la = add_bf16_lo(la, pk[k >> 1]);
-                lb = add_bf16_hi(lb, pk[k >> 1]);
+                    for (int k = 0; k < 8; ++k) o[k] *= f;
+                    tmem_st8(tO + c, reinterpret_cast<const uint32_t*>(o));
+                    tmem_st_wait();   // o is reused
+                  }
+                }
               }
+              const float nref = ref == -INFINITY ? 0.f : -ref;
+              const uint64_t n2 = f2_pack(nref, nref);
+              uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
+              float sq[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+              for (int k = 0; k < 32; k += 2) {
+                float u, v;
+                f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, n2), u, v);
+                u = ex2(u);
+                v = ex2(v);
+                if (k & 2) s2b = f2_add(s2b, f2_pack(u, v));
+                else s2a = f2_add(s2a, f2_pack(u, v));
+                const uint32_t b2 = pack_bf16x2(u, v);
+                pk[k >> 1] = b2;
+                const int c = (k >> 1) & 1;
+                sq[2 * c] = add_bf16_lo(sq[2 * c], b2);
+                sq[2 * c + 1] = add_bf16_hi(sq[2 * c + 1], b2);
+              }
+              float ea, eb, ec, ed;
+              f2_unpack(s2a, ea, eb);
+              f2_unpack(s2b, ec, ed);
+              ls = (ea + eb) + (ec + ed);
+              os = (sq[0] + sq[1]) + (sq[2] + sq[3]);
+              may = me.valid && !(ls <= kMaxChunkSum);
+              if (again || !__any_sync(0xffffffffu, may)) break;
             }
-            tmem_st16(tR + 32 * q2 + 16 * hq, pk);
+            lsum += ls;
+            osum += os;
           }
+          tmem_st16(tR + 16 * q, pk);
         }
         tmem_st_wait();
-        *osum += (la + lb) + (lc + ld);
-        float ea, eb, ec, ed;
-        f2_unpack(s2a, ea, eb);
-        f2_unpack(s2b, ec, ed);
-        return (ea + eb) + (ec + ed);
       };
       auto release = [&]() {   // the warpgroup's columns are read
         tc_fence_before();
@@ -413,6 +462,7 @@ __global__ void __launch_bounds__(kTailThreads, 1)
       };
 
       // ---- rows: query tiles X and X + 2
+#pragma unroll 1
       for (int rr = 0; ok && rr < 2; ++rr) {
         const int qt = X + 2 * rr;
         if (qt >= nq) break;
@@ -420,84 +470,49 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         const Partners me = partners_of(i);
         if (!(ok = tail_wait(&sm.bar_sfull[X], (n_sfull++) & 1, abort_flag))) break;
         tc_fence_after();
-        // half 0: P = exp2(S - max of half 0), exact when there is one half
-        const float m0 = half_max(me, 0, -INFINITY);
-        const float nmc0 = (me.valid && m0 != -INFINITY) ? -m0 * kLogitScale2 : 0.f;
-        float nmc = nmc0;
-        float osum = 0.f;
-        float lsum = half_exp(me, 0, nmc0, &osum);
-        tc_fence_before();
-        warp_arrive(&sm.bar_pready[X]);
-        if (nkh == 2) {
-          // half 1 (at most 128 keys; its S lands on P of half 0 after that
-          // half's P V, so O of half 0 is complete once S is): the reference
-          // rises to its maximum when that exceeds the reference by more than
-          // 8 (base 2, P below 2^8 otherwise), and O and the row sum are
-          // rescaled exactly
-          if (!(ok = tail_wait(&sm.bar_sfull[X], (n_sfull++) & 1, abort_flag))) break;
-          if (!(ok = tail_wait(&sm.bar_odone[X], (n_odone++) & 1, abort_flag))) break;
-          tc_fence_after();
-          const float m1 = half_max(me, 1, -INFINITY);
-          const bool raise = me.valid && m1 != -INFINITY &&
-                             (m0 == -INFINITY || (m1 - m0) * kLogitScale2 > 8.f);
-          float f = 1.f;
-          if (raise) {
-            f = m0 == -INFINITY ? 0.f : ex2((m0 - m1) * kLogitScale2);
-            nmc = -m1 * kLogitScale2;
-            lsum *= f;
-            osum *= f;
-          }
-          if (__any_sync(0xffffffffu, raise)) {
+        float ref = -INFINITY, lsum = 0.f, osum = 0.f;
 #pragma unroll 1
-            for (int c = 0; c < 64; c += 16) {
-              float o[16];
-              tmem_ld16(tO + c, o);
-              tmem_ld_wait();
-#pragma unroll
-              for (int k = 0; k < 16; ++k) o[k] *= f;
-              tmem_st16(tO + c, reinterpret_cast<const uint32_t*>(o));
-              tmem_st_wait();   // o is reused
-            }
+        for (int kh = 0; kh < nkh; ++kh) {
+          if (kh > 0) {
+            // half 1 (at most 128 keys; its S lands on P of half 0 after that
+            // half's P V, so O of half 0 is complete once S is)
+            if (!(ok = tail_wait(&sm.bar_sfull[X], (n_sfull++) & 1, abort_flag))) break;
+            if (!(ok = tail_wait(&sm.bar_odone[X], (n_odone++) & 1, abort_flag))) break;
+            tc_fence_after();
           }
-          lsum += half_exp(me, 1, nmc, &osum);
+          half_softmax(me, kh, ref, lsum, osum);
           tc_fence_before();
           warp_arrive(&sm.bar_pready[X]);
         }
+        if (!ok) break;
+        // rows' -LSE; a valid row attends to itself, so its reference is finite
+        sm.nlse[i] = me.valid ? -(ref + lg2(lsum)) : -INFINITY;
         if (!(ok = tail_wait(&sm.bar_odone[X], (n_odone++) & 1, abort_flag))) break;
         tc_fence_after();
+        if (o_held) store_o();              // the warpgroup's first query tile of two
         const float inv = me.valid ? 1.f / osum : 0.f;
-        float o[64];
-        tmem_ld32(tO, o);
-        tmem_ld32(tO + 32, o + 32);
-        tmem_ld_wait();
-        sm.nlse[i] = me.valid ? -(lg2(lsum) - nmc) : -INFINITY;
-        // O is in registers: the columns may take S^T while O is stored
-        release();
-        // the warp's 32 rows leave in two column halves of 64 bytes (no O
-        // but the last layer's when O is not kept)
-        uint8_t* stage = base + 3 * kTailOpBytes + warp * 2048;
-        uint16_t* const Ol = out_O != nullptr ? out_O + static_cast<size_t>(l) * B * L * H * kHeadDim
-                             : l == n_layers - 1 ? out_O_last : nullptr;
-        uint16_t* row0 =
-            Ol ? Ol + ((static_cast<size_t>(b) * L + i - (r & 31)) * H + h) * kHeadDim : nullptr;
-        const uint32_t rows = __ballot_sync(0xffffffffu, me.valid);
 #pragma unroll
-        for (int c = 0; c < 64 && Ol != nullptr; c += 32) {
+        for (int c = 0; c < 64; c += 32) {
+          float o[32];
+          tmem_ld32(tO + c, o);
+          tmem_ld_wait();
 #pragma unroll
-          for (int k = 0; k < 32; k += 8)
-            stage_row_piece<4>(stage, k >> 3,
-                               make_uint4(pack_bf16x2(o[c + k] * inv, o[c + k + 1] * inv),
-                                          pack_bf16x2(o[c + k + 2] * inv, o[c + k + 3] * inv),
-                                          pack_bf16x2(o[c + k + 4] * inv, o[c + k + 5] * inv),
-                                          pack_bf16x2(o[c + k + 6] * inv, o[c + k + 7] * inv)));
-          flush_staged_rows<4>(stage, row0 + c, static_cast<size_t>(H) * kHeadDim, rows);
+          for (int k = 0; k < 32; k += 2)
+            opk[(c + k) >> 1] = pack_bf16x2(o[k] * inv, o[k + 1] * inv);
         }
+        // O is in registers: the columns may take S^T; O is stored while the
+        // cluster's column sums are awaited
+        release();
+        o_held = true;
+        o_row = i - (r & 31);
+        o_rows = __ballot_sync(0xffffffffu, me.valid);
       }
       // rows past the last query tile take no part in the column sums
       for (int i = kTile * nq + (tid & 255); i < kTailMax; i += 256) sm.nlse[i] = -INFINITY;
       tail_named_sync();   // every LSE is written
 
       // ---- columns: key tiles X and X + 2, summed over the query rows
+#pragma unroll 1
       for (int rr = 0; ok && rr < 2; ++rr) {
         const int kt = X + 2 * rr;
         if (kt >= nq) break;
@@ -508,27 +523,25 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         for (int qh = 0; ok && qh < nkh; ++qh) {
           if (!(ok = tail_wait(&sm.bar_stfull[X], (n_stfull++) & 1, abort_flag))) break;
           tc_fence_after();
-          const int nh = min(256, n - 256 * qh);
-          for (int q2 = 0; q2 < (nh + 63) >> 6; ++q2) {
-            float x[64];
-            tmem_ld32(tST + 64 * q2, x);
-            tmem_ld32(tST + 64 * q2 + 32, x + 32);
+          const int chunks = (min(256, n - 256 * qh) + 31) >> 5;
+#pragma unroll 1
+          for (int q = 0; q < chunks; ++q) {
+            const int qa = 8 * qh + q;   // chunk of query rows
+            const uint32_t in = partner_mask(me, sm, cur, qa, n);
+            if (!__any_sync(0xffffffffu, in != 0u)) continue;   // outside every window
+            float x[32];
+            tmem_ld32(tST + 32 * q, x);
             tmem_ld_wait();
+            apply_mask(x, in);
+            const float* lw = sm.nlse + 32 * qa;
 #pragma unroll
-            for (int hq = 0; hq < 2; ++hq) {
-              const int qa = 8 * qh + 2 * q2 + hq;   // chunk of query rows
-              float* xh = x + 32 * hq;
-              apply_mask(xh, partner_mask(me, sm, cur, qa, n));
-              const float* lw = sm.nlse + 32 * qa;
-#pragma unroll
-              for (int k = 0; k < 32; k += 4) {
-                const float4 l4 = *reinterpret_cast<const float4*>(lw + k);
-                float e0, e1, e2, e3;
-                f2_unpack(f2_fma(f2_pack(xh[k], xh[k + 1]), c2, f2_pack(l4.x, l4.y)), e0, e1);
-                f2_unpack(f2_fma(f2_pack(xh[k + 2], xh[k + 3]), c2, f2_pack(l4.z, l4.w)), e2, e3);
-                a2a = f2_add(a2a, f2_pack(ex2(e0), ex2(e1)));
-                a2b = f2_add(a2b, f2_pack(ex2(e2), ex2(e3)));
-              }
+            for (int k = 0; k < 32; k += 4) {
+              const float4 l4 = *reinterpret_cast<const float4*>(lw + k);
+              float e0, e1, e2, e3;
+              f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, f2_pack(l4.x, l4.y)), e0, e1);
+              f2_unpack(f2_fma(f2_pack(x[k + 2], x[k + 3]), c2, f2_pack(l4.z, l4.w)), e2, e3);
+              a2a = f2_add(a2a, f2_pack(ex2(e0), ex2(e1)));
+              a2b = f2_add(a2b, f2_pack(ex2(e2), ex2(e3)));
             }
           }
           if (nq > 1) release();
@@ -540,30 +553,34 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         // cluster barrier below (release / acquire) makes it visible there
         const float cs = me.valid ? (a0 + a2) + (a1 + a3) : 0.f;
         const uint32_t la = smem_u32(colall + (par * kTailMaxHeads + h) * kTailMax + j);
+#pragma unroll 4
         for (int hh = 0; hh < H; ++hh) st_dsmem_f32(dsmem_addr(la, hh), cs);
       }
     }
 
     // ------------------------------------------------- heads, threshold, compaction
     tc_fence_before();
-    cluster_sync();
+    cluster_arrive();
+    if (o_held) store_o();
+    cluster_wait_acquire();
     tc_fence_after();
     const int nxt = cur ^ 1;
     if (tid < 256) {
+      const int rounds = n > 256 ? 2 : 1;   // tokens tid and tid + 256
       float sj[2] = {0.f, 0.f};
+      const float inv_hn = static_cast<float>(H * n);
 #pragma unroll
       for (int rd = 0; rd < 2; ++rd) {
         const int j = tid + 256 * rd;
-        if (j < n) {
+        if (rd < rounds && j < n) {
           const float* cj = colall + par * kTailMaxHeads * kTailMax + j;
           float v[kTailMaxHeads];
 #pragma unroll
           for (int hh = 0; hh < kTailMaxHeads; ++hh) v[hh] = hh < H ? cj[hh * kTailMax] : 0.f;
           float a = 0.f;
 #pragma unroll
-          for (int hh = 0; hh < kTailMaxHeads; ++hh)
-            if (hh < H) a += v[hh];
-          sj[rd] = a / static_cast<float>(H * n);
+          for (int hh = 0; hh < kTailMaxHeads; ++hh) a += v[hh];   // (zeros past H)
+          sj[rd] = a / inv_hn;
           if (h == 0) out_scores[(static_cast<size_t>(l) * B + b) * L + j] = sj[rd];
         }
       }
@@ -603,45 +620,34 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         const uint32_t kb = __ballot_sync(0xffffffffu, keep[rd]);
         if (lane == 0) sm.kbits[rd][warp] = kb;
       }
+      if (tid < kTailChunks) sm.gbits[nxt][tid] = 0u;
       tail_named_sync();
-      // every thread reads the 16 ballot words (round-major, then warp) and
-      // forms its own exclusive prefix and the total
-      int kpre[2] = {0, 0}, total = 0;
-      {
-        const uint4* kw = reinterpret_cast<const uint4*>(&sm.kbits[0][0]);
+      // lane k holds ballot word k (round-major, then warp) and its prefix
+      const uint32_t word = lane < 16 ? (&sm.kbits[0][0])[lane] : 0u;
+      int upto = __popc(word);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint4 u = kw[q];
-          const uint32_t wv[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int idx = 4 * q + e;   // = 8 * round + warp
-            if (idx == warp) kpre[0] = total;
-            if (idx == 8 + warp) kpre[1] = total;
-            total += __popc(wv[e]);
-          }
-        }
+      for (int off = 1; off < 16; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, upto, off);
+        if (lane >= off) upto += y;
       }
+      const int total = __shfl_sync(0xffffffffu, upto, 15);
 #pragma unroll
       for (int rd = 0; rd < 2; ++rd) {
+        if (rd >= rounds) break;
+        const uint32_t mine = __shfl_sync(0xffffffffu, word, 8 * rd + warp);
+        const int before = __shfl_sync(0xffffffffu, upto, 8 * rd + warp) - __popc(mine);
         if (!keep[rd]) continue;
         const int j = tid + 256 * rd;
-        const int k = kpre[rd] + __popc(sm.kbits[rd][warp] & ((1u << lane) - 1u));
+        const int k = before + __popc(mine & ((1u << lane) - 1u));
         const int ps = sm.pos[cur][j];
         sm.pos[nxt][k] = ps;
+        if ((sm.gbits[cur][j >> 5] >> (j & 31)) & 1u)
+          atomicOr(&sm.gbits[nxt][k >> 5], 1u << (k & 31));
         if (h == 0) out_pos[(static_cast<size_t>(l + 1) * B + b) * L + k] = ps;
       }
       if (tid == 0) {
         sm.n[nxt] = total;
         if (h == 0) out_len[static_cast<size_t>(l + 1) * B + b] = total;
-      }
-      tail_named_sync();
-#pragma unroll
-      for (int rd = 0; rd < 2; ++rd) {
-        const int k = tid + 256 * rd;
-        const bool gk = k < total && tail_is_global(sm, sm.pos[nxt][k]);
-        const uint32_t gb = __ballot_sync(0xffffffffu, gk);
-        if (lane == 0 && (k >> 5) < kTailChunks) sm.gbits[nxt][k >> 5] = gb;
       }
     }
     cur = nxt;
