@@ -59,6 +59,7 @@ constexpr uint32_t kTailDyn = 3 * kTailOpBytes + kTailStageBytes + kTailColBytes
 static_assert(kTailDyn > 233472 / 2, "the tail kernel must occupy an SM alone");
 
 struct TailSmem {
+  uint64_t bar_cols[2];               // every head's column sums of a layer (by parity) are here
   uint64_t bar_sfull[2], bar_sfree[2], bar_pready[2], bar_odone[2], bar_stfull[2], bar_fin[2];
   uint32_t tmem_base;
   int abort;
@@ -169,6 +170,7 @@ __global__ void __launch_bounds__(kTailThreads, 1)
     reinterpret_cast<uint4*>(base)[k] = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) {
     for (int X = 0; X < 2; ++X) {
+      mbar_init(&sm.bar_cols[X], 1);
       mbar_init(&sm.bar_sfull[X], 1);
       mbar_init(&sm.bar_sfree[X], 4);   // one arrival per warp
       mbar_init(&sm.bar_pready[X], 4);
@@ -217,6 +219,8 @@ __global__ void __launch_bounds__(kTailThreads, 1)
     const int nq = (n + kTile - 1) / kTile;   // 128-row tiles (1..3)
     const int nkh = n > 256 ? 2 : 1;          // key (query) halves of at most 256
     const int par = it & 1;
+    if (tid == 0)   // what the heads' CTAs send for this layer
+      mbar_arrive_expect_tx(&sm.bar_cols[par], static_cast<uint32_t>(H * n) * 4u);
 
     // ---- rows of the current tokens: 16-byte pieces, 128B-swizzled tiles
     {
@@ -549,26 +553,27 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         float a0, a1, a2, a3;
         f2_unpack(a2a, a0, a1);
         f2_unpack(a2b, a2, a3);
-        // this head's sum of column j goes to every CTA of the cluster; the
-        // cluster barrier below (release / acquire) makes it visible there
-        const float cs = me.valid ? (a0 + a2) + (a1 + a3) : 0.f;
-        const uint32_t la = smem_u32(colall + (par * kTailMaxHeads + h) * kTailMax + j);
+        // this head's sum of column j goes to every CTA of the cluster, counted
+        // there.  (A CTA is at most one layer ahead of another, whose sums of the
+        // layer between it has to wait for: the two buffers suffice.)
+        const float cs = (a0 + a2) + (a1 + a3);
+        const uint32_t la = smem_u32(colall + (par * kTailMaxHeads + h) * kTailMax + j),
+                       lb = smem_u32(&sm.bar_cols[par]);
+        if (me.valid)
 #pragma unroll 4
-        for (int hh = 0; hh < H; ++hh) st_dsmem_f32(dsmem_addr(la, hh), cs);
+          for (int hh = 0; hh < H; ++hh) st_async_f32(dsmem_addr(la, hh), cs, dsmem_addr(lb, hh));
       }
     }
 
     // ------------------------------------------------- heads, threshold, compaction
-    tc_fence_before();
-    cluster_arrive();
     if (o_held) store_o();
-    cluster_wait_acquire();
-    tc_fence_after();
+    tc_fence_before();
     const int nxt = cur ^ 1;
     if (tid < 256) {
       const int rounds = n > 256 ? 2 : 1;   // tokens tid and tid + 256
       float sj[2] = {0.f, 0.f};
       const float inv_hn = static_cast<float>(H * n);
+      __all_sync(0xffffffffu, mbar_wait_cluster(&sm.bar_cols[par], (it >> 1) & 1, abort_flag));
 #pragma unroll
       for (int rd = 0; rd < 2; ++rd) {
         const int j = tid + 256 * rd;

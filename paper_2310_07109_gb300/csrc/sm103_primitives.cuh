@@ -493,6 +493,38 @@ __device__ __forceinline__ void st_dsmem_f32(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
+// A store into another CTA's shared memory that counts its 4 bytes on an mbarrier
+// there once it is visible to whoever waits for that barrier (both addresses in
+// the cluster's shared window).
+__device__ __forceinline__ void st_async_f32(uint32_t addr, float v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr),
+               "r"(__float_as_uint(v)), "r"(bar)
+               : "memory");
+}
+
+// Bounded wait for a barrier on which other CTAs of the cluster count stores.
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity,
+                                                  volatile int* abort) {
+  const uint32_t t0 = global_timer_lo();
+#pragma unroll 1
+  for (;;) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (*abort) return false;
+    if (global_timer_lo() - t0 > 2000000000u) {
+      *abort = 1;
+      return false;
+    }
+  }
+}
+
 // 16-byte global -> shared copy through the load/store path (no register
 // staging); completes at cp_async_wait_all().  Writes via the generic proxy.
 __device__ __forceinline__ void cp_async16(uint32_t saddr, const void* gptr) {
