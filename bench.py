@@ -534,16 +534,24 @@ def run_native(args, wl):
     value = whole_job_rate(world, kept_per_step, ms_per_step)
 
     # ---- kernels launched per timed step.  A captured step, and an eager call
-    # (which the library records into a graph of its own), runs the per-layer
-    # kernels in a device-driven loop: prep, [padding gather], rows + cols +
-    # gather + advance for each layer that some sequence still runs per layer
-    # (more than TAIL_MAX_LEN tokens), then the cluster kernel.  With plain
-    # launches: the library's plan.
+    # (which the library records into a graph of its own): prep, [padding
+    # gather], then rows + scores + gather for every layer that the arguments
+    # let need them, or, where they do not tell, rows + scores + gather + advance
+    # for layer 0 and for pairs of later layers while some sequence has more than
+    # TAIL_MAX_LEN tokens, then the cluster kernel.  With plain launches: the
+    # library's plan.
     eager_launches = sc.stack_launch_count(wl.n_layers, wl.B, wl.L, wl.H, wl.w, gpos,
                                            inp["pad_mask"] is not None)
     looped = sum(1 for l in range(wl.n_layers) if (lens[l] > sc.TAIL_MAX_LEN).any())
-    graph_launches = (1 + (1 if inp["pad_mask"] is not None else 0) + 4 * looped + 1
-                      if wl.L > sc.TAIL_MAX_LEN else 2)
+    pad = 1 if inp["pad_mask"] is not None else 0
+    if wl.L <= sc.TAIL_MAX_LEN:
+        graph_launches = 2
+    elif wl.keep_rule == sc.SC_KEEP_TOP_RATIO:
+        graph_launches = 1 + pad + 3 * looped - 1 + 1   # no gather after the last
+    elif all(a <= 0 for a in wl.alphas()[:-1]):
+        graph_launches = 1 + pad + 3 * wl.n_layers - 1 + pad
+    else:
+        graph_launches = 1 + pad + 4 * (1 + 2 * ((looped - 1 + 1) // 2)) + 1
     launches_per_step = (eager_launches if graph is None and args.plain_launches
                          else graph_launches)
 
@@ -603,7 +611,7 @@ def run_native(args, wl):
     if rows_ms[0] + cols_ms[0] > 1e-6:
         unit_bytes, unit_flops, unit_t = work[0][0], work[0][1], t_l0
         unit_kernels = ["sc_rows_kernel", "sc_cols_kernel"]
-        unit_desc = ("sc_rows_kernel + sc_cols_kernel of layer 0 (one launch each, chained "
+        unit_desc = ("sc_rows_kernel + sc_scores_kernel of layer 0 (one launch each, chained "
                      "as in the timed step; B=%d sequences of %d tokens)"
                      % (wl.B, int(lens[0].max())))
     else:

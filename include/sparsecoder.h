@@ -241,8 +241,11 @@ int sc_layer_forward(const sc_layer_args* args, void* workspace, size_t workspac
  * (within the stated tolerances).
  *
  * Launches: in a CUDA graph (a call made while `stream` is being captured)
- * the per-layer kernels run in a loop whose condition the device sets, so
- * the layers that every sequence runs in the cluster kernel launch nothing.
+ * the per-layer kernels run in a loop whose condition the device sets (two
+ * layers a turn), so the layers that every sequence runs in the cluster kernel
+ * launch nothing; where the arguments bound the layers that can need the
+ * per-layer kernels (the top-ratio rule; thresholds <= 0 in every layer but the
+ * last), just those are launched, without a loop.
  * An eager call (stream not capturing) that has both kinds of kernels in its
  * plan runs the same way: the library records the call into a graph of its
  * own, keeps the instantiated graph (up to 16 per process, least recently
@@ -276,9 +279,10 @@ int sc_stack_forward_profiled(const sc_stack_args* args, void* workspace, size_t
 /* Number of kernels that sc_stack_forward launches for these arguments (on the
  * current device) when it launches them directly (SC_STACK_PLAIN_LAUNCHES, or
  * a plan with one kind of kernel), in *count.  A call that runs as a graph
- * launches prep, [padding-removal gather], then rows, cols, gather and a
- * loop-advance kernel for layer 0 and for each later layer that some sequence
- * still runs per layer, then the cluster kernel.  Only the sizes, n_layers,
+ * launches prep, [padding-removal gather], then rows, scores and gather for each
+ * layer whose need the arguments bound, or rows, scores, gather and a
+ * loop-advance kernel for layer 0 and for pairs of later layers while some
+ * sequence still runs per layer, then the cluster kernel.  Only the sizes, n_layers,
  * flags, pad_mask (NULL or not) and the global list are read; no pointer is
  * dereferenced and nothing is launched.  Errors: see sc_status (SC_ERR_CUDA
  * without a usable device). */

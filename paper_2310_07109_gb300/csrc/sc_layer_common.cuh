@@ -84,14 +84,15 @@ __device__ __forceinline__ LayerView layer_view(const LayerParams& p) {
   v.ident_out = odd ? const_cast<int32_t*>(p.ident) : p.ident_out;
   v.O = p.O != nullptr ? p.O + l * p.o_stride : (l == p.n_layers - 1 ? p.O_last : nullptr);
   v.scores = p.scores + l * p.row_stride;
-  v.alpha = p.alphas[l];
+  v.alpha = p.alphas[min(l, kTailMaxLayers - 1)];
   return v;
 }
 
-// Sequence b has been handed to the cluster kernel for this and later layers
-// (its length here may be stale: read nothing else of it).
+// Sequence b has been handed to the cluster kernel for this and later layers, or
+// the device-driven loop is past the last layer (its length here may be stale:
+// read nothing else of it).
 __device__ __forceinline__ bool owned_by_tail(const LayerParams& p, const LayerView& v, int b) {
-  return p.tail_from != nullptr && __ldcg(p.tail_from + b) <= v.layer;
+  return p.tail_from != nullptr && (v.layer >= p.n_layers || __ldcg(p.tail_from + b) <= v.layer);
 }
 
 // Which source holds the current rows of sequence b, and the token index of

@@ -1,0 +1,71 @@
+"""Stacks whose arguments bound the layers that need the per-layer kernels (the
+top-ratio rule, thresholds that nothing can miss) record those layers without
+the device-driven loop, and other stacks take two layers per turn of it: the
+results are those of the plain launches bit for bit, and nothing past a length
+is written."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+RELATIVE, ABSOLUTE, TOP_RATIO = 0, 1, 2
+CASES = [
+    # layers, L, lens (None: no padding), rule, alphas
+    (5, 700, None, TOP_RATIO, [0.9] * 5),                     # 700 ... 459, 414, then 372
+    (5, 700, [700, 385, 384, 1], TOP_RATIO, [0.9] * 5),
+    (4, 900, None, TOP_RATIO, [1.0, 0.4, 1.0, 1.0]),
+    (1, 500, None, TOP_RATIO, [0.5]),
+    (4, 500, None, RELATIVE, [0.0] * 4),
+    (4, 500, [500, 400, 200, 37], RELATIVE, [0.0, -1.0, 0.0, 0.7]),   # the last alpha prunes
+    (3, 640, [640, 1, 384, 385], ABSOLUTE, [-1.0, 0.0, 5.0]),
+    (2, 700, None, RELATIVE, [0.0, 0.9]),
+    # not bounded: the loop, left after an odd and an even number of layers
+    (4, 700, None, RELATIVE, [0.3, 0.0, 0.0, 0.0]),
+    (5, 700, [700, 500, 100, 650], RELATIVE, [0.1, 0.9, 0.9, 0.9, 0.9]),
+    (6, 700, None, RELATIVE, [1e-3] * 6),                     # nothing pruned, 6 layers
+    (7, 700, None, RELATIVE, [1e-3] * 7),
+]
+
+
+@pytest.mark.parametrize("host", [False, True])
+@pytest.mark.parametrize("nl,L,lens,rule,alphas", CASES)
+def test_graph_equals_plain_launches(nl, L, lens, rule, alphas, host):
+    import paper_2310_07109_gb300 as sc
+    B, H = 4, 4
+    g = torch.Generator(device="cuda")
+    g.manual_seed(L + nl)
+    Q, K, V = (torch.randn((nl, B, L, H, 64), device="cuda", generator=g).bfloat16()
+               for _ in range(3))
+    mask = None
+    if lens is not None:
+        mask = (torch.arange(L)[None, :] < torch.tensor(lens)[:, None]).to(torch.uint8).cuda()
+    if host:
+        Q, K, V = (t.cpu().pin_memory() for t in (Q, K, V))
+        mask = mask if mask is None else mask.cpu().pin_memory()
+
+    def call(plain):
+        if host:
+            out = sc.new_host_outputs(nl, B, L, H)
+            ws = sc.new_stack_host_workspace(nl, B, L, H)
+        else:
+            out = {"O": torch.empty((nl, B, L, H, 64), dtype=torch.bfloat16, device="cuda"),
+                   "scores": torch.empty((nl, B, L), device="cuda"),
+                   "pos": torch.empty((nl + 1, B, L), dtype=torch.int32, device="cuda"),
+                   "len": torch.empty((nl + 1, B), dtype=torch.int32, device="cuda")}
+            ws = sc.new_workspace(B, L, H)
+        for t in out.values():
+            t.fill_(7)
+        fn = sc.stack_forward_host if host else sc.stack_forward
+        fn(Q, K, V, mask, [0, 5, L // 2], 64, alphas, out=out, workspace=ws, keep_rule=rule,
+           plain_launches=plain)
+        torch.cuda.synchronize()
+        assert sc.workspace_status(ws) == 0
+        return {k: t.cpu() for k, t in out.items()}
+
+    a, b = call(False), call(True)
+    for k in a:
+        x, y = (t[k].view(torch.int16) if k == "O" else t[k] for t in (a, b))
+        if lens is None and rule != TOP_RATIO and not host and all(v <= 0 for v in alphas[:-1]):
+            # every layer stays with the per-layer kernels in both (nothing gets short)
+            assert int(a["len"][:-1].min()) == L
+        assert torch.equal(x, y), k
