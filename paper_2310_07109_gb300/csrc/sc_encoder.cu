@@ -14,9 +14,10 @@
 // projection (Y is the next layer's X, already compacted).
 //
 // GEMM: output tiles of 128 rows of one sequence (rows are (sequence, row)
-// pairs, row < rows[b] read on the device) by 256, 192 or 128 columns (chosen
-// on the host), one persistent CTA per SM walking the tiles; K in steps of 64
-// through a four-stage TMA ring: A's 128 rows by one tiled copy, or by
+// pairs, row < rows[b] read on the device) by 256, 192, 128 or 64 columns (chosen
+// on the device from the rows there are), one persistent CTA per SM walking the
+// tiles that hold rows; K in steps of 64 through a TMA ring of four to eight
+// stages: A's 128 rows by one tiled copy, or by
 // four-row gathers (tile::gather4, any row order) when A is gathered, W's rows
 // by one tiled copy, both 128B-swizzled and K-major; one thread issues the
 // MMAs (M = 128) into one of two 256-column fp32 accumulators in tensor memory
@@ -34,29 +35,48 @@ namespace sc {
 
 constexpr int kGemmThreads = 320;   // warp 0 loads, warp 1 issues, warps 2-9 write back
 constexpr int kGemmEpiWarps = 8;    // two per tensor-memory lane quarter, one column half each
-constexpr int kGemmStages = 4;
+constexpr int kGemmMinStages = 4;   // ring stages of 256-column tiles
+constexpr int kGemmMaxStages = 8;   // ... of 64-column tiles, in the same shared memory
+constexpr int kGemmMinBN = 64;      // narrowest tile
+constexpr int kGemmSeqs = 128;      // most sequences whose tiles are counted out
 constexpr int kGemmBK = 64;         // K per stage: one 128-byte swizzle atom of bf16
 constexpr int kGemmBN = 256;        // most output columns per tile (one MMA, N <= 256)
 constexpr uint32_t kGemmABytes = kTileBytes;              // 128 rows x 64
 constexpr uint32_t kGemmWBytes = kGemmBN * kGemmBK * 2;   // 256 rows x 64
-constexpr uint32_t kGemmStageBytes = kGemmABytes + kGemmWBytes;
+constexpr uint32_t kGemmRingBytes = kGemmMinStages * (kGemmABytes + kGemmWBytes);
 // after the ring: a 4 KB staging area per write-back warp (32 rows of 128 bytes),
 // through which the stores of a chunk leave as whole row segments
 constexpr uint32_t kGemmStageOut = 4096;
-constexpr uint32_t kGemmDyn = kGemmStages * kGemmStageBytes + kGemmEpiWarps * kGemmStageOut + 1024;
+constexpr uint32_t kGemmDyn = kGemmRingBytes + kGemmEpiWarps * kGemmStageOut + 1024;
 
 struct GemmSmem {
-  uint64_t full[kGemmStages], empty[kGemmStages];
+  uint64_t full[kGemmMaxStages], empty[kGemmMaxStages];
   uint64_t tfull[2], tempty[2];   // accumulator buffers: written by the MMAs, read back
   uint32_t tmem_base;
   int abort;
+  // per sequence: row tiles of the sequences before it (up to all), its rows
+  int tile0[kGemmSeqs + 1];
+  int rows[kGemmSeqs];
+  int bn;
 };
+
+static_assert(sizeof(GemmSmem) + kGemmDyn <= 227 * 1024, "one CTA's shared memory");
 
 // Bounded wait that ignores the abort flag (teardown: no copy or MMA may still
 // write into this CTA's memory when it exits).
 __device__ __forceinline__ void drain_wait_gemm(uint64_t* bar, uint32_t parity) {
   int dummy = 0;
   mbar_wait(bar, parity, &dummy, 1000000000ull);
+}
+
+// Nothing may still be landing in shared memory when the CTA exits: the last
+// fill of every stage.  `use` rounds of the ring and s stages have been filled.
+__device__ __forceinline__ void gemm_drain_full(GemmSmem& sm, int stages, int s, int use) {
+#pragma unroll 1
+  for (int q = 0; q < stages; ++q) {
+    const int fills = use + (q < s ? 1 : 0);
+    if (fills > 0) drain_wait_gemm(&sm.full[q], (fills - 1) & 1);
+  }
 }
 
 __device__ __forceinline__ bool warp_wait_gemm(uint64_t* bar, uint32_t parity, volatile int* abort) {
@@ -94,24 +114,81 @@ __device__ __forceinline__ void gelu_erf2(float& x0, float& x1) {
 }
 
 // Tile t of the launch: column block nt of width bn (fastest, so that the
-// CTAs of a wave share A rows), row tile rt of sequence b.
+// CTAs of a wave share A rows), row tile rt of sequence b.  Where the tiles that
+// hold rows are counted out (rows given, at most kGemmSeqs sequences) t counts
+// only these; a role's tiles come in increasing order, so `b` is advanced.
 struct GemmTile {
   int b, r0, n0, nw, rows;
   bool skip;
 };
 
-__device__ __forceinline__ GemmTile gemm_tile(const GemmParams& p, int t) {
-  const int tiles_n = (p.N + p.bn - 1) / p.bn;
-  const int tiles_r = (p.L + kTile - 1) / kTile;
-  GemmTile g;
+__device__ __forceinline__ bool gemm_counted(const GemmParams& p) {
+  return p.rows != nullptr && p.B <= kGemmSeqs;
+}
+
+__device__ __forceinline__ void gemm_tile(const GemmParams& p, const GemmSmem& sm, int bn, int t,
+                                          GemmTile& g) {
+  const int tiles_n = (p.N + bn - 1) / bn;
   const int nt = t % tiles_n, rest = t / tiles_n;
-  g.b = rest / tiles_r;
-  g.r0 = (rest % tiles_r) * kTile;
-  g.n0 = nt * p.bn;
-  g.nw = min(p.bn, p.N - g.n0);
-  g.rows = p.rows ? min(__ldcg(p.rows + g.b), p.L) : p.L;
+  if (gemm_counted(p)) {
+    while (sm.tile0[g.b + 1] <= rest) ++g.b;
+    g.r0 = (rest - sm.tile0[g.b]) * kTile;
+    g.rows = sm.rows[g.b];
+  } else {
+    const int tiles_r = (p.L + kTile - 1) / kTile;
+    g.b = rest / tiles_r;
+    g.r0 = (rest % tiles_r) * kTile;
+    g.rows = p.rows ? min(__ldcg(p.rows + g.b), p.L) : p.L;
+  }
+  g.n0 = nt * bn;
+  g.nw = min(bn, p.N - g.n0);
   g.skip = g.r0 >= g.rows;
-  return g;
+}
+
+// Counts out the row tiles of every sequence and chooses the tile width; warp 0.
+__device__ __forceinline__ void gemm_plan(const GemmParams& p, GemmSmem& sm, int lane) {
+  int total = p.B * ((p.L + kTile - 1) / kTile);
+  if (gemm_counted(p)) {
+    total = 0;
+#pragma unroll 1
+    for (int b0 = 0; b0 < p.B; b0 += 32) {
+      const int b = b0 + lane;
+      const int n = b < p.B ? min(__ldcg(p.rows + b), p.L) : 0;
+      int x = (max(n, 0) + kTile - 1) / kTile;   // inclusive scan
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += y;
+      }
+      if (b < p.B) {
+        sm.rows[b] = n;
+        sm.tile0[b + 1] = total + x;
+      }
+      total += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) sm.tile0[0] = 0;
+  }
+  // The width with the least (whole rounds of tiles over the CTAs) x (width + 32),
+  // the 32 a per-tile cost in columns' worth of time: the tiles run in rounds of
+  // one per SM, so a width that leaves a last round mostly empty costs a whole
+  // round.  Widths divide N and the split blocks; with a gathered A, 256 (A is
+  // fetched again for every column tile).  One width per lane.  A short batch
+  // leaves most SMs idle and each busy one fetches at its own L2 rate, so there
+  // the narrowest tiles win: a layer of one sequence of 200 tokens takes 67.5 us
+  // with 64-column tiles and 77.2 with 128 as the narrowest.  Counting the rows
+  // that are there, not the L there may be, gives a layer of 8 x 1024 tokens with
+  // a third pruned 198 us instead of 212.
+  uint32_t key = 0xffffffffu;
+  const int c = kGemmBN - 64 * lane;
+  if (c > 0 && (p.a_idx == nullptr || c == kGemmBN)) {
+    const bool fits = p.N % c == 0 && (p.out_split <= 0 || p.out_split % c == 0);
+    const uint32_t tiles = static_cast<uint32_t>(total) * ((p.N + c - 1) / c);
+    const uint32_t cost = (tiles + gridDim.x - 1) / gridDim.x * (c + 32);
+    if (fits) key = min(cost, 0x0fffffffu) * 4 + lane;
+    else if (c == kGemmBN) key = 0xfffffff0u;   // where nothing fits: masked last columns
+  }
+  key = __reduce_min_sync(0xffffffffu, key);
+  if (lane == 0) sm.bn = kGemmBN - 64 * static_cast<int>(key & 3);
 }
 
 // Persistent: each CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...;
@@ -119,18 +196,15 @@ __device__ __forceinline__ GemmTile gemm_tile(const GemmParams& p, int t) {
 // write-back of one tile overlaps the MMAs of the next.
 __global__ void __launch_bounds__(kGemmThreads, 1)
     sc_gemm_kernel(const __grid_constant__ GemmParams p) {
-  pdl_wait();
-  pdl_launch_dependents();
   extern __shared__ uint8_t dyn_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dyn_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   __shared__ GemmSmem sm;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ksteps = p.K / kGemmBK;
-  const int tiles = p.B * ((p.L + kTile - 1) / kTile) * ((p.N + p.bn - 1) / p.bn);
 
   if (tid == 0) {
-    for (int s = 0; s < kGemmStages; ++s) {
+    for (int s = 0; s < kGemmMaxStages; ++s) {
       mbar_init(&sm.full[s], 1);
       mbar_init(&sm.empty[s], 1);
     }
@@ -142,80 +216,110 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     fence_mbar_init();
   }
   if (warp == 1) tmem_alloc(&sm.tmem_base, 512);
+  // what the launch before this one writes is read from here on
+  pdl_wait();
+  pdl_launch_dependents();
+  if (warp == 0) gemm_plan(p, sm, lane);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tm = sm.tmem_base;
   volatile int* abort_flag = &sm.abort;
+  const int bn = sm.bn;
+  // A's rows and W's of one K step; as many stages as the ring holds (4 to 8)
+  const uint32_t stage_bytes = kGemmABytes + bn * kGemmBK * 2;
+  const int stages = min(kGemmMaxStages, static_cast<int>(kGemmRingBytes / stage_bytes));
+  const int tiles = (gemm_counted(p) ? sm.tile0[p.B] : p.B * ((p.L + kTile - 1) / kTile)) *
+                    ((p.N + bn - 1) / bn);
+  GemmTile g;
+  g.b = 0;
 
   if (warp == 0) {
     // ------------------------------------------------------------- loads
+    const CUtensorMap* map_w = &p.map_w[bn / 64 - 1];
+    const uint32_t w_bytes = min(bn, p.N) * kGemmBK * 2;   // rows past N: zeros
     bool ok = true;
     int s = 0, use = 0;
-    for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
-      const GemmTile g = gemm_tile(p, t);
-      if (g.skip) continue;
-      // gathered A: this lane's four rows (rows past the sequence read row 0:
-      // discarded); otherwise one tiled copy of 128 consecutive rows
-      int ar[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int r = g.r0 + 4 * lane + k;
-        const int src =
-            r < g.rows ? (p.a_idx ? __ldcg(p.a_idx + static_cast<size_t>(g.b) * p.L + r) : r) : 0;
-        ar[k] = g.b * p.L + src;
-      }
-      const bool gather = p.a_idx != nullptr;
-      for (int kt = 0; ok && kt < ksteps; ++kt) {
-        if (use > 0 && !(ok = warp_wait_gemm(&sm.empty[s], (use - 1) & 1, abort_flag))) break;
-        uint8_t* As = base + s * kGemmStageBytes;
-        uint8_t* Ws = As + kGemmABytes;
-        if (lane == 0) {
-          mbar_arrive_expect_tx(&sm.full[s], kGemmABytes + p.wbox * kGemmBK * 2);
-          tma_load_2d(Ws, &p.map_w, kt * kGemmBK, g.n0, &sm.full[s]);
-          if (!gather) tma_load_2d(As, &p.map_at, kt * kGemmBK, g.b * p.L + g.r0, &sm.full[s]);
+    if (p.a_idx == nullptr) {
+      // one lane: a tiled copy of 128 consecutive rows, and one of W's rows (a
+      // second W copy per step would cost 190 cycles: this loop paces short calls)
+      if (elect_one()) {
+        for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
+          gemm_tile(p, sm, bn, t, g);
+          if (g.skip) continue;
+          const int row = g.b * p.L + g.r0;
+#pragma unroll 1
+          for (int kt = 0; kt < ksteps; ++kt) {
+            if (use > 0 && !(ok = mbar_wait(&sm.empty[s], (use - 1) & 1, abort_flag))) break;
+            uint8_t* As = base + s * stage_bytes;
+            mbar_arrive_expect_tx(&sm.full[s], kGemmABytes + w_bytes);
+            tma_load_2d(As + kGemmABytes, map_w, kt * kGemmBK, g.n0, &sm.full[s]);
+            tma_load_2d(As, &p.map_a, kt * kGemmBK, row, &sm.full[s]);
+            if (++s == stages) {
+              s = 0;
+              ++use;
+            }
+          }
         }
-        __syncwarp();
-        if (gather)
+        gemm_drain_full(sm, stages, s, use);
+      }
+    } else {
+      for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
+        gemm_tile(p, sm, bn, t, g);
+        if (g.skip) continue;
+        // this lane's four rows (rows past the sequence read row 0: discarded)
+        int ar[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int r = g.r0 + 4 * lane + k;
+          ar[k] = g.b * p.L +
+                  (r < g.rows ? __ldcg(p.a_idx + static_cast<size_t>(g.b) * p.L + r) : 0);
+        }
+#pragma unroll 1
+        for (int kt = 0; kt < ksteps; ++kt) {
+          if (use > 0 && !(ok = warp_wait_gemm(&sm.empty[s], (use - 1) & 1, abort_flag))) break;
+          uint8_t* As = base + s * stage_bytes;
+          if (lane == 0) {
+            mbar_arrive_expect_tx(&sm.full[s], kGemmABytes + w_bytes);
+            tma_load_2d(As + kGemmABytes, map_w, kt * kGemmBK, g.n0, &sm.full[s]);
+          }
+          __syncwarp();
           tma_gather4(As + 512 * lane, &p.map_a, kt * kGemmBK, ar[0], ar[1], ar[2], ar[3],
                       &sm.full[s]);
-        if (++s == kGemmStages) {
-          s = 0;
-          ++use;
+          if (++s == stages) {
+            s = 0;
+            ++use;
+          }
         }
       }
+      if (lane == 0) gemm_drain_full(sm, stages, s, use);
     }
-    // nothing may still be landing in shared memory when the CTA exits: the
-    // last fill of every slot
-    if (lane == 0)
-      for (int q = 0; q < kGemmStages; ++q) {
-        const int fills = use + (q < s ? 1 : 0);
-        if (fills > 0) drain_wait_gemm(&sm.full[q], (fills - 1) & 1);
-      }
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------- MMA issue
-    if (lane == 0) {
+    if (elect_one()) {
       bool ok = true;
       int s = 0, use = 0, j = 0;
+      const uint32_t ring = smem_u32(base);
       for (int t = blockIdx.x; ok && t < tiles; t += gridDim.x) {
-        const GemmTile g = gemm_tile(p, t);
+        gemm_tile(p, sm, bn, t, g);
         if (g.skip) continue;
         const int acc = j & 1;
         // the buffer's previous tile has been read back
-        if (j >= 2 && !(ok = mbar_wait(&sm.tempty[acc], ((j >> 1) - 1) & 1, abort_flag))) break;
+        if (j >= 2 && !(ok = mbar_wait(&sm.tempty[acc], ((j >> 1) - 1) & 1, abort_flag)))
+          break;
         tc_fence_after();
-        const uint32_t idesc = idesc_bf16(128, g.nw, false, false);
-        const uint32_t d = tm + acc * kGemmBN;
-        for (int kt = 0; ok && kt < ksteps; ++kt) {
+        const uint32_t d = tm + acc * kGemmBN, idesc = idesc_bf16(128, g.nw, false, false);
+#pragma unroll 1
+        for (int kt = 0; kt < ksteps; ++kt) {
           if (!(ok = mbar_wait(&sm.full[s], use & 1, abort_flag))) break;
           tc_fence_after();
-          const uint32_t a = smem_u32(base + s * kGemmStageBytes), w = a + kGemmABytes;
+          const uint32_t a = sdesc_lo(ring + s * stage_bytes), w = a + (kGemmABytes >> 4);
 #pragma unroll
           for (int k = 0; k < kGemmBK / 16; ++k)
-            umma_bf16(d, sdesc_sw128(a + 32 * k), sdesc_sw128(w + 32 * k), idesc, (kt | k) != 0);
+            umma_bf16_lo(d, a + 2 * k, w + 2 * k, idesc, (kt | k) != 0);
           umma_commit(&sm.empty[s]);   // the stage is free once these MMAs are done
-          if (++s == kGemmStages) {
+          if (++s == stages) {
             s = 0;
             ++use;
           }
@@ -224,11 +328,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         ++j;
       }
       // every MMA has completed before the tensor memory is freed
-      uint64_t* last = &sm.empty[(s + kGemmStages - 1) % kGemmStages];
       if (use > 0 || s > 0) {
-        const int q = (s + kGemmStages - 1) % kGemmStages;
+        const int q = (s + stages - 1) % stages;
         const int fills = use + (q < s ? 1 : 0);
-        drain_wait_gemm(last, (fills - 1) & 1);
+        drain_wait_gemm(&sm.empty[q], (fills - 1) & 1);
       }
     }
     __syncwarp();
@@ -236,11 +339,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     // ------------------------------------------------------------- write back
     const int q = warp & 3;                  // tensor-memory lane quarter of this warp
     const int ch = (warp - 2) / 4;           // column half of the tile
-    uint8_t* const stg = base + kGemmStages * kGemmStageBytes + (warp - 2) * kGemmStageOut;
+    uint8_t* const stg = base + kGemmRingBytes + (warp - 2) * kGemmStageOut;
     bool ok = true;
     int j = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
-      const GemmTile g = gemm_tile(p, t);
+      gemm_tile(p, sm, bn, t, g);
       if (g.skip) continue;
       const int acc = j & 1;
       const int r = g.r0 + 32 * q + lane;
@@ -249,7 +352,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
           in_rows ? (p.res_idx ? __ldcg(p.res_idx + static_cast<size_t>(g.b) * p.L + r) : r) : 0;
       const uint16_t* res =
           p.res ? p.res + (static_cast<size_t>(g.b) * p.L + rsrc) * p.N + g.n0 : nullptr;
-      const int cbeg = ch * (p.bn / 2), cend = min(g.nw, (ch + 1) * (p.bn / 2));
+      const int cbeg = ch * (bn / 2), cend = min(g.nw, (ch + 1) * (bn / 2));
       // without GELU, this row's residual over the warp's first two chunks of
       // 32 columns is loaded before the accumulator is ready, so that its
       // latency overlaps the MMAs (later chunks, and GEMMs with GELU, load
@@ -510,8 +613,9 @@ cudaError_t launch_gemm(const GemmParams& p, cudaStream_t st) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
   }
+  const int least = p.a_idx != nullptr ? kGemmBN : kGemmMinBN;   // narrowest tiles possible
   const long long tiles = static_cast<long long>(p.B) * ((p.L + kTile - 1) / kTile) *
-                          ((p.N + p.bn - 1) / p.bn);
+                          ((p.N + least - 1) / least);
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);
   return launch_pdl(sc_gemm_kernel, dim3(grid), dim3(kGemmThreads), kGemmDyn, st, p);
 }
