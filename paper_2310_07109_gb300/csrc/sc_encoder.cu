@@ -26,7 +26,6 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <cstdint>
-#include <type_traits>
 
 #include "sc_internal.cuh"
 #include "sm103_primitives.cuh"
@@ -34,7 +33,8 @@
 namespace sc {
 
 constexpr int kGemmThreads = 320;   // warp 0 loads, warp 1 issues, warps 2-9 write back
-constexpr int kGemmEpiWarps = 8;    // two per tensor-memory lane quarter, one column half each
+constexpr int kGemmEpiWarps = 8;    // two per tensor-memory lane quarter, every other chunk
+constexpr int kGemmChunkStep = 32 * (kGemmEpiWarps / 4);   // columns between a warp's chunks
 constexpr int kGemmMinStages = 4;   // ring stages of 256-column tiles
 constexpr int kGemmMaxStages = 8;   // ... of 64-column tiles, in the same shared memory
 constexpr int kGemmMinBN = 64;      // narrowest tile
@@ -54,10 +54,11 @@ struct GemmSmem {
   uint64_t tfull[2], tempty[2];   // accumulator buffers: written by the MMAs, read back
   uint32_t tmem_base;
   int abort;
-  // per sequence: row tiles of the sequences before it (up to all), its rows
+  // per sequence: row tiles of the sequences before it (up to all)
   int tile0[kGemmSeqs + 1];
-  int rows[kGemmSeqs];
+  uint8_t pad[kGemmSeqs];   // rows missing in the last tile
   int bn;
+  alignas(16) float bias[kGemmBN];   // of the tile being written back
 };
 
 static_assert(sizeof(GemmSmem) + kGemmDyn <= 227 * 1024, "one CTA's shared memory");
@@ -81,6 +82,11 @@ __device__ __forceinline__ void gemm_drain_full(GemmSmem& sm, int stages, int s,
 
 __device__ __forceinline__ bool warp_wait_gemm(uint64_t* bar, uint32_t parity, volatile int* abort) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
+}
+
+// The write-back warps meet (barrier 1).
+__device__ __forceinline__ void gemm_sync_epilogue() {
+  asm volatile("bar.sync 1, %0;" ::"n"(32 * kGemmEpiWarps) : "memory");
 }
 
 __device__ __forceinline__ uint16_t bf16_bits(float x) {
@@ -133,7 +139,7 @@ __device__ __forceinline__ void gemm_tile(const GemmParams& p, const GemmSmem& s
   if (gemm_counted(p)) {
     while (sm.tile0[g.b + 1] <= rest) ++g.b;
     g.r0 = (rest - sm.tile0[g.b]) * kTile;
-    g.rows = sm.rows[g.b];
+    g.rows = (sm.tile0[g.b + 1] - sm.tile0[g.b]) * kTile - sm.pad[g.b];
   } else {
     const int tiles_r = (p.L + kTile - 1) / kTile;
     g.b = rest / tiles_r;
@@ -153,15 +159,15 @@ __device__ __forceinline__ void gemm_plan(const GemmParams& p, GemmSmem& sm, int
 #pragma unroll 1
     for (int b0 = 0; b0 < p.B; b0 += 32) {
       const int b = b0 + lane;
-      const int n = b < p.B ? min(__ldcg(p.rows + b), p.L) : 0;
-      int x = (max(n, 0) + kTile - 1) / kTile;   // inclusive scan
+      const int n = b < p.B ? max(min(__ldcg(p.rows + b), p.L), 0) : 0;
+      int x = (n + kTile - 1) / kTile;   // inclusive scan
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, x, off);
         if (lane >= off) x += y;
       }
       if (b < p.B) {
-        sm.rows[b] = n;
+        sm.pad[b] = static_cast<uint8_t>(-n & (kTile - 1));
         sm.tile0[b + 1] = total + x;
       }
       total += __shfl_sync(0xffffffffu, x, 31);
@@ -194,6 +200,10 @@ __device__ __forceinline__ void gemm_plan(const GemmParams& p, GemmSmem& sm, int
 // Persistent: each CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...;
 // the accumulator alternates between two 256-column buffers, so that the
 // write-back of one tile overlaps the MMAs of the next.
+// kPlain: bf16 out without a residual.  The fp32 staging and the residual are
+// another instance: with both in one, the write-back loop of a feed-forward
+// product with GELU (8 x 1024 rows, 768 -> 3072) took 45.2 us, without 38.5.
+template <bool kPlain>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     sc_gemm_kernel(const __grid_constant__ GemmParams p) {
   extern __shared__ uint8_t dyn_raw[];
@@ -337,8 +347,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     __syncwarp();
   } else {
     // ------------------------------------------------------------- write back
+    // This part paces the products with K = 768: the copies of the next tile fill
+    // the L2 ports, so anything it loads on the way costs up to a microsecond a
+    // chunk.  Hence the bias through shared memory, the residual two chunks ahead
+    // and in the layout of the stores (one row per lane touched 32 lines a load),
+    // and one rolled loop.  8 x 1024 rows: 768 -> 2304 30.1 -> 24.4 us,
+    // 768 -> 3072 with GELU 52.3 -> 38.6, 768 -> 768 with residual 22.1 -> 18.2.
+    // Sixteen warps were slower (27.4, 50.1, 22.8).
     const int q = warp & 3;                  // tensor-memory lane quarter of this warp
-    const int ch = (warp - 2) / 4;           // column half of the tile
+    const int c0 = (warp - 2) / 4 * 32;      // its first chunk of 32 columns
+    const int et = tid - 64;
     uint8_t* const stg = base + kGemmRingBytes + (warp - 2) * kGemmStageOut;
     bool ok = true;
     int j = 0;
@@ -348,26 +366,31 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
       const int acc = j & 1;
       const int r = g.r0 + 32 * q + lane;
       const bool in_rows = r < g.rows;
-      const int rsrc =
-          in_rows ? (p.res_idx ? __ldcg(p.res_idx + static_cast<size_t>(g.b) * p.L + r) : r) : 0;
-      const uint16_t* res =
-          p.res ? p.res + (static_cast<size_t>(g.b) * p.L + rsrc) * p.N + g.n0 : nullptr;
-      const int cbeg = ch * (bn / 2), cend = min(g.nw, (ch + 1) * (bn / 2));
-      // without GELU, this row's residual over the warp's first two chunks of
-      // 32 columns is loaded before the accumulator is ready, so that its
-      // latency overlaps the MMAs (later chunks, and GEMMs with GELU, load
-      // theirs chunk by chunk)
-      const bool res_ahead = res != nullptr && !p.gelu;
-      uint4 rpf[2][4];
+      // the residual of a chunk as the lanes store it (four columns of rows
+      // lane / 8 + 4 k), loaded two chunks ahead: under the copies of the products
+      // a load takes up to a microsecond
+      [[maybe_unused]] uint2 rv[2][8];
+      [[maybe_unused]] int rsrc = 0;
+      [[maybe_unused]] auto load_res = [&](uint2 (&to)[8], int c) {
+        if (p.res == nullptr || c >= g.nw) return;
+        const uint16_t* res =
+            p.res + static_cast<size_t>(g.b) * p.L * p.N + g.n0 + 4 * (lane & 7) + c;
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int c = cbeg + 32 * u;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          rpf[u][k] = (res_ahead && c < cend)
-                          ? __ldcg(reinterpret_cast<const uint4*>(res + c + 8 * k))
-                          : make_uint4(0u, 0u, 0u, 0u);
+        for (int k = 0; k < 8; ++k) {
+          const int row = __shfl_sync(0xffffffffu, rsrc, 4 * k + lane / 8);
+          to[k] = __ldcg(reinterpret_cast<const uint2*>(res + static_cast<size_t>(row) * p.N));
+        }
+      };
+      if constexpr (!kPlain) {
+        if (in_rows) rsrc = p.res_idx ? __ldcg(p.res_idx + static_cast<size_t>(g.b) * p.L + r) : r;
+        load_res(rv[0], c0);
+        load_res(rv[1], c0 + kGemmChunkStep);
       }
+      // the tile's bias, once every warp is done with the previous one's
+      const float bias = p.bias && et < g.nw ? __ldg(p.bias + g.n0 + et) : 0.f;
+      gemm_sync_epilogue();
+      if (et < kGemmBN) sm.bias[et] = bias;
+      gemm_sync_epilogue();
       ok = ok && warp_wait_gemm(&sm.tfull[acc], (j >> 1) & 1, abort_flag);
       const uint32_t rows_mask = __ballot_sync(0xffffffffu, ok && in_rows);
       const size_t orow0 = static_cast<size_t>(g.b) * p.L + g.r0 + 32 * q;   // the warp's row 0
@@ -380,52 +403,26 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         ldo = p.out_split;
       }
       tc_fence_after();
-      // one 32-column chunk: bias, GELU (only where may_gelu is true), the
-      // residual (rv: its 32 values, or nullptr: loaded here), store
-      auto chunk = [&](int c, const uint4* rv, auto may_gelu) {
+#pragma unroll 1
+      for (int c = c0; rows_mask != 0u && c < g.nw; c += kGemmChunkStep) {
         float v[32];
         tmem_ld32(tm + acc * kGemmBN + (static_cast<uint32_t>(32 * q) << 16) + c, v);
         tmem_ld_wait();
-        if (rows_mask == 0u) return;   // warp-uniform
-        const float4* bp = reinterpret_cast<const float4*>(p.bias + g.n0 + c);
+        const float4* bp = reinterpret_cast<const float4*>(sm.bias + c);
 #pragma unroll
         for (int k = 0; k < 32; k += 4) {
-          const float4 b4 = p.bias ? __ldg(bp + k / 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 b4 = bp[k / 4];
           v[k] += b4.x;
           v[k + 1] += b4.y;
           v[k + 2] += b4.z;
           v[k + 3] += b4.w;
         }
-        if constexpr (decltype(may_gelu)::value) {
-          if (p.gelu)
+        if (p.gelu)
 #pragma unroll
-            for (int k = 0; k < 32; k += 2) gelu_erf2(v[k], v[k + 1]);
-        }
-        if (res != nullptr) {
-#pragma unroll
-          for (int k = 0; k < 32; k += 8) {
-            const uint4 r4 = rv != nullptr ? rv[k / 8]
-                                           : __ldcg(reinterpret_cast<const uint4*>(res + c + k));
-            const uint32_t w4[4] = {r4.x, r4.y, r4.z, r4.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              v[k + 2 * e] += __uint_as_float(w4[e] << 16);
-              v[k + 2 * e + 1] += __uint_as_float(w4[e] & 0xffff0000u);
-            }
-          }
-        }
-        // the warp's 32 rows leave as whole 128-byte (fp32) or 64-byte (bf16)
-        // row segments; rows past the sequence are not written
-        if (p.out_f32) {
-#pragma unroll
-          for (int k = 0; k < 32; k += 4)
-            stage_row_piece<8>(stg, k / 4,
-                               make_uint4(__float_as_uint(v[k]), __float_as_uint(v[k + 1]),
-                                          __float_as_uint(v[k + 2]), __float_as_uint(v[k + 3])));
-          flush_staged_rows<8>(
-              stg, reinterpret_cast<uint16_t*>(static_cast<float*>(outp) + orow0 * ldo + nb + c),
-              2 * static_cast<size_t>(ldo), rows_mask);
-        } else {
+          for (int k = 0; k < 32; k += 2) gelu_erf2(v[k], v[k + 1]);
+        // the warp's 32 rows leave as row segments of 128 bytes (fp32) or 64 (bf16);
+        // rows past the sequence are not written
+        if constexpr (kPlain) {
 #pragma unroll
           for (int k = 0; k < 32; k += 8)
             stage_row_piece<4>(stg, k / 8,
@@ -434,16 +431,36 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                                           pack_bf16x2(v[k + 6], v[k + 7])));
           flush_staged_rows<4>(stg, static_cast<uint16_t*>(outp) + orow0 * ldo + nb + c,
                                static_cast<size_t>(ldo), rows_mask);
+          continue;
         }
-      };
-      if (!res_ahead) {
-#pragma unroll 1
-        for (int c = cbeg; c < cend; c += 32) chunk(c, nullptr, std::true_type{});
-      } else {
-        // unrolled, so that the prefetched residual stays in registers
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (cbeg + 32 * u < cend) chunk(cbeg + 32 * u, u < 2 ? rpf[u] : nullptr, std::false_type{});
+        for (int k = 0; k < 32; k += 4)
+          stage_row_piece<8>(stg, k / 4,
+                             make_uint4(__float_as_uint(v[k]), __float_as_uint(v[k + 1]),
+                                        __float_as_uint(v[k + 2]), __float_as_uint(v[k + 3])));
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int rr = 4 * k + lane / 8;
+          float4 o = *reinterpret_cast<const float4*>(stg + stage_offset<8>(rr, lane & 7));
+          if (p.res != nullptr) {
+            o.x += __uint_as_float(rv[0][k].x << 16);
+            o.y += __uint_as_float(rv[0][k].x & 0xffff0000u);
+            o.z += __uint_as_float(rv[0][k].y << 16);
+            o.w += __uint_as_float(rv[0][k].y & 0xffff0000u);
+            rv[0][k] = rv[1][k];
+          }
+          if ((rows_mask >> rr) & 1u) {
+            const size_t at = (orow0 + rr) * ldo + nb + c + 4 * (lane & 7);
+            if (p.out_f32)
+              *reinterpret_cast<float4*>(static_cast<float*>(outp) + at) = o;
+            else
+              *reinterpret_cast<uint2*>(static_cast<uint16_t*>(outp) + at) =
+                  make_uint2(pack_bf16x2(o.x, o.y), pack_bf16x2(o.z, o.w));
+          }
+        }
+        load_res(rv[1], c + 2 * kGemmChunkStep);
+        __syncwarp();   // the staging area may be written again
       }
       // the buffer may take the tile after next
       tc_fence_before();
@@ -585,7 +602,11 @@ __global__ void __launch_bounds__(kLnThreads)
 // launch helpers used by the C ABI
 // ---------------------------------------------------------------------------
 cudaError_t configure_encoder() {
-  return cudaFuncSetAttribute(sc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e =
+      cudaFuncSetAttribute(sc_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(kGemmDyn));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(sc_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(kGemmDyn));
 }
 
@@ -617,7 +638,7 @@ cudaError_t launch_gemm(const GemmParams& p, cudaStream_t st) {
   const long long tiles = static_cast<long long>(p.B) * ((p.L + kTile - 1) / kTile) *
                           ((p.N + least - 1) / least);
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);
-  return launch_pdl(sc_gemm_kernel, dim3(grid), dim3(kGemmThreads), kGemmDyn, st, p);
+  return launch_pdl(p.res == nullptr && !p.out_f32 ? sc_gemm_kernel<true> : sc_gemm_kernel<false>, dim3(grid), dim3(kGemmThreads), kGemmDyn, st, p);
 }
 
 cudaError_t launch_row_gather(const RowGatherParams& p, cudaStream_t st) {

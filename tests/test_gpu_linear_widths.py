@@ -41,3 +41,29 @@ def test_linear_widths(sc, B, L, rows, N, K):  # noqa: F811
     # fp32 sums of K exact products: the bar of the other fp32 outputs
     np.testing.assert_allclose(got[used], want[used], rtol=0, atol=1e-4 * np.abs(want).max())
     assert np.isnan(got[~used]).all(), "rows past the sequence were written"
+
+
+@pytest.mark.parametrize("gelu,out_f32", [(False, True), (True, False), (True, True)])
+def test_linear_residual_of_four_chunks(sc, gelu, out_f32):  # noqa: F811
+    """Gathered rows keep 256-column tiles: a write-back warp takes four chunks of
+    the residual, two loaded before the product is there and two on the way."""
+    rng = np.random.default_rng(3)
+    B, L, N, K, n = 2, 150, 384, 128, np.array([150, 131], np.int32)
+    A = _bf16(rng.standard_normal((B * L, K)))
+    W = _bf16(rng.standard_normal((N, K)) / math.sqrt(K))
+    R = _bf16(rng.standard_normal((B * L, N)))
+    gidx = np.stack([rng.permutation(L) for _ in range(B)]).astype(np.int32)
+    out = torch.full((B * L, N), float("nan"), device="cuda",
+                     dtype=torch.float32 if out_f32 else torch.bfloat16)
+    sc.linear_forward(_t_bf16(A), _t_bf16(W), B=B, L=L, rows=torch.from_numpy(n).cuda(),
+                      gidx=torch.from_numpy(gidx).cuda(), gelu=gelu, res=_t_bf16(R),
+                      res_gathered=True, out=out, out_f32=out_f32)
+    got = out.float().cpu().numpy().astype(np.float64)
+    for b in range(B):
+        src = b * L + gidx[b, :n[b]]
+        y = enc.linear(A[src], W, np.zeros(N))
+        y = (enc.gelu(y) if gelu else y) + R[src]
+        # bf16 out: half an ulp, 2^-9 |y|, and as much again for the fp32 part
+        tol = (1e-4 * np.abs(y).max(), 0) if out_f32 else (1e-4, 2.0 ** -8)
+        np.testing.assert_allclose(got[b * L:b * L + n[b]], y, atol=tol[0], rtol=tol[1])
+        assert np.isnan(got[b * L + n[b]:(b + 1) * L]).all()
