@@ -36,7 +36,7 @@ struct BlockSync {
 // flags come from the cut over all n scores, found here (`scratch`: shared
 // memory the CTA no longer uses, for the selection's histogram and tie flags).
 template <int kThreads>
-__device__ void finalize_sequence(const LayerParams& p, const LayerView& v, int b, int n,
+__device__ void finalize_sequence(const LayerParams& p, const LayerView& v, int b, int n, int ng,
                                   FinalSmem<kThreads>& sm, const int* gc, uint8_t* scratch) {
   constexpr int kRounds = FinalSmem<kThreads>::kRounds;
   constexpr int kWarps = kThreads / 32;
@@ -118,7 +118,6 @@ __device__ void finalize_sequence(const LayerParams& p, const LayerView& v, int 
     if (out == sm.total - 1) sm.last_pos = ps[r];
   }
   // next-layer index of each surviving global token
-  const int ng = min(__ldcg(v.ng + b), kMaxGlobal);
   if (tid < ng) {
     const int c = gc[tid], r = c / kThreads, t = c % kThreads;
     const uint32_t bits = sm.kbits[r][t >> 5];

@@ -1234,7 +1234,7 @@ __global__ void __launch_bounds__(kColsThreads, 2)
   __syncthreads();
   if (!sm.flag) return;
   __threadfence();
-  finalize_sequence<kColsThreads>(p, v, b, n, sm.fin, sm.gc, base);
+  finalize_sequence<kColsThreads>(p, v, b, n, ng, sm.fin, sm.gc, base);
 }
 
 // ---------------------------------------------------------------------------

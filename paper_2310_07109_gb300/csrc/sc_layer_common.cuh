@@ -13,14 +13,6 @@
 
 namespace sc {
 
-// ---------------------------------------------------------------------------
-// small helpers
-// ---------------------------------------------------------------------------
-// Barrier over the four warps of softmax warpgroup X (ids 2 and 3).
-__device__ __forceinline__ void named_sync_wg(int X) {
-  asm volatile("bar.sync %0, 128;" ::"r"(2 + X) : "memory");
-}
-
 __device__ __forceinline__ void named_sync_softmax() {
   asm volatile("bar.sync 1, 128;" ::: "memory");
 }

@@ -22,6 +22,10 @@ CASES = [
     (700, [700, 130], 0, [0, 350], 2.0),
     (700, [700], 64, [0, 699], 40.0),                          # references raised by far
     (640, [640], 639, [5], 40.0),
+    # scores: factors found by a thread per (head, global row), rows in batches of
+    # four after the first, more key tiles than one batch of them
+    (300, [300, 129], 64, list(range(0, 300, 19)), 2.0),       # 16 globals, two head blocks
+    (1200, [1200, 1025], 100, [0, 3, 200, 600, 1024, 1199], 2.0),
 ]
 
 
