@@ -18,7 +18,8 @@
 //            key column j the sum over rows of exp2(S_ij - LSE_i): one thread
 //            per column, no cross-thread sums
 //   heads    each CTA writes its column sums into every CTA of the cluster
-//            (distributed shared memory) before the cluster barrier; every CTA
+//            (st.async, counted in bytes on a barrier of the receiver, so that no
+//            CTA waits for more than the sums it adds); every CTA
 //            then adds the heads in the same fixed order, so all
 //            take the same keep decisions (s_j >= alpha_l / n, j == 0 kept) and
 //            compact the token list the same way, without a second exchange
@@ -46,14 +47,13 @@ constexpr int kTailTiles = (kTailMax + kTile - 1) / kTile;   // 128-row tiles (3
 constexpr uint32_t kTailOpBytes = kTailTiles * kTileBytes;   // rows of one tensor (48 KB)
 constexpr int kTailChunks = kTailMax / 32;                    // 32-token chunks (12)
 static_assert(kTailMax <= 384, "a second key half must fit beside O in tensor memory");
-constexpr float kMaxChunkSum = 16777216.f;                   // 2^24 (see half_softmax)
 constexpr uint32_t kTailStageBytes = 8 * 2048;                // O row staging, 2 KB per softmax warp
 // column sums of every head, [layer parity][head][column], written by the
 // CTA of that head into every CTA of the cluster
 constexpr uint32_t kTailColBytes = 2 * kTailMaxHeads * kTailMax * 4;
 // Q, K, V operands, the O staging and alignment; more than half of an SM's
 // shared memory, so a second CTA never shares the SM (each holds all 512
-// tensor-memory columns while it waits at cluster barriers: two CTAs of
+// tensor-memory columns while it waits for its cluster: two CTAs of
 // different clusters on one SM could otherwise wait on each other's allocation).
 constexpr uint32_t kTailDyn = 3 * kTailOpBytes + kTailStageBytes + kTailColBytes + 1024;
 static_assert(kTailDyn > 233472 / 2, "the tail kernel must occupy an SM alone");
@@ -350,14 +350,17 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         me.all = w >= n - 1 || ((sm.gbits[cur][i >> 5] >> (i & 31)) & 1u);
         return me;
       };
-      // Softmax of half kh (S in tensor memory) against the row's reference, 32
-      // keys at a time: P = exp2(S - ref), written as bf16 pairs over the first
-      // half of the columns (each chunk's pairs land on columns that this or an
-      // earlier chunk has read).  The reference is the maximum of the first chunk
-      // that the row attends to; a chunk whose exponentials sum to more than
-      // kMaxChunkSum raises it by a whole power of two, by which everything
-      // formed so far (the half's P, the sums, and O of the half before) is
-      // scaled exactly.
+      // Softmax of half kh (S in tensor memory), 32 keys at a time, in two passes:
+      // the row's maximum over the half, then P = exp2(S - ref), written as bf16
+      // pairs over the first half of the columns (each chunk's pairs land on
+      // columns that this or an earlier chunk has read).  The reference is the
+      // maximum of half 0 (so the largest P of a row is 1, which bf16 holds
+      // exactly); half 1 raises it to its own maximum when that lies more than 8
+      // above, O and the sums being rescaled.  The first pass writes the scores
+      // back masked, and the second neither masks nor looks at windows again: a
+      // 12-layer stack of 16 x 333 tokens takes 275 us so, 292 with the masks
+      // applied twice, and 273 with a reference from the first chunk alone, which
+      // made O's error against 64 bits 2 to 4 % larger.
       // lsum: the sum of the exponentials (fp32: the row's LSE, which the column
       // sums use); osum: the sum of the same values rounded to the bf16 that P V
       // multiplies (the normaliser of O, so that O is a weighted mean of V rows
@@ -366,95 +369,88 @@ __global__ void __launch_bounds__(kTailThreads, 1)
       // to stay in the instruction caches.
       auto half_softmax = [&](const Partners& me, int kh, float& ref, float& lsum, float& osum) {
         const int chunks = (round16(min(256, n - 256 * kh)) + 31) >> 5;
+        float mx = -INFINITY;
+        uint32_t some = 0u;   // chunks inside some row's window (warp-uniform)
 #pragma unroll 1
         for (int q = 0; q < chunks; ++q) {
           const uint32_t in = partner_mask(me, sm, cur, 8 * kh + q, n);
+          if (!__any_sync(0xffffffffu, in != 0u)) continue;
+          some |= 1u << q;
+          float x[32];
+          tmem_ld32(tR + 32 * q, x);
+          tmem_ld_wait();
+          if (!__all_sync(0xffffffffu, in == 0xffffffffu)) {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) x[k] = ((in >> k) & 1u) ? x[k] : -INFINITY;
+            tmem_st32(tR + 32 * q, x);   // masked: the second pass takes it as it is
+          }
+          float m2 = -INFINITY;
+#pragma unroll
+          for (int k = 0; k < 32; k += 4) {
+            mx = fmax3(mx, x[k], x[k + 1]);
+            m2 = fmax3(m2, x[k + 2], x[k + 3]);
+          }
+          mx = fmaxf(mx, m2);
+        }
+        tmem_st_wait();
+        mx *= kLogitScale2;
+        if (kh == 0) {
+          ref = mx;
+        } else {
+          const bool raise = mx > ref + 8.f;
+          if (__any_sync(0xffffffffu, raise)) {
+            float f = 1.f;
+            if (raise) {
+              f = ref == -INFINITY ? 0.f : ex2(ref - mx);
+              ref = mx;
+              lsum *= f;
+              osum *= f;
+            }
+#pragma unroll 1
+            for (int c = 0; c < 64; c += 8) {
+              float o[8];
+              tmem_ld8(tO + c, o);
+              tmem_ld_wait();
+#pragma unroll
+              for (int k = 0; k < 8; ++k) o[k] *= f;
+              tmem_st8(tO + c, reinterpret_cast<const uint32_t*>(o));
+              tmem_st_wait();   // o is reused
+            }
+          }
+        }
+        const float nref = ref == -INFINITY ? 0.f : -ref;
+        const uint64_t n2 = f2_pack(nref, nref);
+#pragma unroll 1
+        for (int q = 0; q < chunks; ++q) {
           uint32_t pk[16];
-          if (!__any_sync(0xffffffffu, in != 0u)) {   // outside every row's window
+          if (((some >> q) & 1u) == 0u) {   // outside every row's window
 #pragma unroll
             for (int k = 0; k < 16; ++k) pk[k] = 0u;
           } else {
             float x[32];
             tmem_ld32(tR + 32 * q, x);
             tmem_ld_wait();
-            apply_mask(x, in);
-            float ls, os;
-            bool may = in != 0u && ref == -INFINITY;
-#pragma unroll 1
-            for (bool again = false;; again = true) {   // again: under a raised reference
-              if (__any_sync(0xffffffffu, may)) {
-                float mx = -INFINITY;
+            uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
+            float sq[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int k = 0; k < 32; k += 2) mx = fmax3(mx, x[k], x[k + 1]);
-                mx *= kLogitScale2;
-                float f = 1.f;
-                if (may && mx > ref + 8.f) {
-                  if (ref == -INFINITY) {   // all sums and P so far are 0
-                    ref = mx;
-                  } else {
-                    const float up = ceilf(mx - ref);
-                    f = ex2(-up);
-                    ref += up;
-                    lsum *= f;
-                    osum *= f;
-                  }
-                }
-                if (__any_sync(0xffffffffu, f != 1.f)) {
-#pragma unroll 1
-                  for (int c = 0; c < 16 * q; c += 8) {
-                    float w8[8];
-                    tmem_ld8(tR + c, w8);
-                    tmem_ld_wait();
-                    uint32_t u[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                      const uint32_t b2 = __float_as_uint(w8[k]);
-                      u[k] = pack_bf16x2(__uint_as_float(b2 << 16) * f,
-                                         __uint_as_float(b2 & 0xffff0000u) * f);
-                    }
-                    tmem_st8(tR + c, u);
-                    tmem_st_wait();
-                  }
-#pragma unroll 1
-                  for (int c = 0; kh > 0 && c < 64; c += 8) {
-                    float o[8];
-                    tmem_ld8(tO + c, o);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) o[k] *= f;
-                    tmem_st8(tO + c, reinterpret_cast<const uint32_t*>(o));
-                    tmem_st_wait();   // o is reused
-                  }
-                }
-              }
-              const float nref = ref == -INFINITY ? 0.f : -ref;
-              const uint64_t n2 = f2_pack(nref, nref);
-              uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
-              float sq[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-              for (int k = 0; k < 32; k += 2) {
-                float u, v;
-                f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, n2), u, v);
-                u = ex2(u);
-                v = ex2(v);
-                if (k & 2) s2b = f2_add(s2b, f2_pack(u, v));
-                else s2a = f2_add(s2a, f2_pack(u, v));
-                const uint32_t b2 = pack_bf16x2(u, v);
-                pk[k >> 1] = b2;
-                const int c = (k >> 1) & 1;
-                sq[2 * c] = add_bf16_lo(sq[2 * c], b2);
-                sq[2 * c + 1] = add_bf16_hi(sq[2 * c + 1], b2);
-              }
-              float ea, eb, ec, ed;
-              f2_unpack(s2a, ea, eb);
-              f2_unpack(s2b, ec, ed);
-              ls = (ea + eb) + (ec + ed);
-              os = (sq[0] + sq[1]) + (sq[2] + sq[3]);
-              may = me.valid && !(ls <= kMaxChunkSum);
-              if (again || !__any_sync(0xffffffffu, may)) break;
+            for (int k = 0; k < 32; k += 2) {
+              float u, v;
+              f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, n2), u, v);
+              u = ex2(u);
+              v = ex2(v);
+              if (k & 2) s2b = f2_add(s2b, f2_pack(u, v));
+              else s2a = f2_add(s2a, f2_pack(u, v));
+              const uint32_t b2 = pack_bf16x2(u, v);
+              pk[k >> 1] = b2;
+              const int c = (k >> 1) & 1;
+              sq[2 * c] = add_bf16_lo(sq[2 * c], b2);
+              sq[2 * c + 1] = add_bf16_hi(sq[2 * c + 1], b2);
             }
-            lsum += ls;
-            osum += os;
+            float ea, eb, ec, ed;
+            f2_unpack(s2a, ea, eb);
+            f2_unpack(s2b, ec, ed);
+            lsum += (ea + eb) + (ec + ed);
+            osum += (sq[0] + sq[1]) + (sq[2] + sq[3]);
           }
           tmem_st16(tR + 16 * q, pk);
         }
