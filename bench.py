@@ -16,8 +16,8 @@ norms, feed-forward on the kept tokens; random-init weights) on the config-2
 shape.  Each prints its own line.
 
 One step = one call of sc_stack_forward over the whole workload: padding removal,
-then per layer the rows kernel (band + global attention, O, row LSE) and the
-cols kernel (column scores, threshold, compaction), 12 layers, inputs resident in
+then per layer the rows kernel (band + global attention, O, column sums) and the
+scores kernel (scores, threshold, compaction), 12 layers, inputs resident in
 HBM.  The default workload is the 12-layer stack B=2, L=4096, H=12, d=64, window
 +-256, token 0 plus 8 seeded global positions, 5% salient keys x4, alpha 0.4->1.0.
 The inputs of one step (453 MB of Q/K/V) are larger than the 129 MB L2, so no
@@ -581,9 +581,9 @@ def run_native(args, wl):
     cols_ms /= prof_steps
     gath_ms /= prof_steps
     prep_ms /= prof_steps
-    # layer 0's rows and cols kernels as one unit, chained as in an
-    # uninstrumented step (no event between them: the cols CTAs of the heads
-    # whose rows are done run beside the rows kernel's last CTAs)
+    # layer 0's rows and scores kernels as one unit, chained as in an
+    # uninstrumented step (no event between them: the scores CTAs of the
+    # sequences whose rows are done run beside the rows kernel's last CTAs)
     pair_ev = [None] * nev
     pair_ev[1] = torch.cuda.Event(enable_timing=True)
     pair_ev[3] = torch.cuda.Event(enable_timing=True)

@@ -651,8 +651,8 @@ static int stack_forward_impl(const sc_stack_args* a, void* workspace, size_t ws
     gp.dst[t] = cmp[t];
   }
   // Host buffers: layer 0's rows cross the host link; the gather walks them
-  // sequence by sequence and counts what it has copied, and layer 0's rows and
-  // cols kernels start on a sequence as soon as its rows are in.
+  // sequence by sequence and counts what it has copied, and layer 0's
+  // attention kernels start on a sequence as soon as its rows are in.
   uint32_t* const gathered = host_io ? reinterpret_cast<uint32_t*>(ws + lay.gathered) : nullptr;
   const uint32_t gather_target = static_cast<uint32_t>((a->L + 7) / 8);
   if (dev_loop) {

@@ -96,7 +96,7 @@ struct LayerParams {
   uint32_t* cols_done;   // [B][H]: cols CTAs of (sequence, head) whose global-row parts are stored
   // nonzero: the gather kernel before this launch is still copying later
   // sequences' rows when it starts: sequence b's rows are complete once
-  // gathered[b] reaches gather_target (the rows and cols kernels wait for it
+  // gathered[b] reaches gather_target (the attention kernels wait for it
   // instead of for the whole gather grid)
   const uint32_t* gathered;
   uint32_t gather_target;

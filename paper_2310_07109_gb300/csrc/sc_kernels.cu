@@ -82,11 +82,11 @@ constexpr uint32_t kPgBlock = 2 * 1024;
 // each pass, and about eight further issue slots; with one softmax warp of each
 // CTA on an SM sub-partition the in-order issue of two warps (IPC 0.4 of 1),
 // not the exponential unit (a fifth busy) or the tensor cores (a quarter).  So
-// the gains lie in instructions and latencies: no maximum in an ordinary item,
-// three items in flight, narrow bands by 64-key items and 32-column chunks,
-// two independent CTAs.  Code size counts as much: every section but the two
-// item loops runs once a CTA, and at 78 KB of code instead of 55 KB the
-// kernel missed the instruction caches and took 14% longer.
+// the gains lie in instructions and latencies: three items in flight, narrow
+// bands by 64-key items and 32-column chunks, two independent CTAs.  Code size
+// counts as much: every section but the two item loops runs once a CTA, and at
+// 78 KB of code instead of 55 KB the kernel missed the instruction caches and
+// took 14% longer.
 // Layer 0 of 2 x 4096 tokens (w 256, 12 heads, 9 global tokens), rows and scores
 // together: 81 us, against 89 us for pairs of query tiles in one CTA per SM
 // with whole-tile items and a tensor-core scores kernel; 4 x 4096: 113 against
@@ -98,7 +98,7 @@ constexpr int kBufs = 3;
 constexpr int kHalf = 64;                        // columns of a buffer: keys (queries) of an item
 constexpr uint32_t kColO = kBufs * kHalf;
 constexpr uint32_t kColPG = kMaxGlobal;          // P_G in its buffer, after S_G
-constexpr float kMaxItemSum = 16777216.f;        // 2^24
+constexpr float kRefSlack = 6.f;                 // base 2 (see the softmax)
 
 struct RowsSmem {
   alignas(16) float nlse[kTile];         // -LSE of the tile's rows (read as float4)
@@ -530,44 +530,51 @@ __global__ void __launch_bounds__(kRowsThreads, 2)
     };
 
     // Softmax with a running reference m_ref (base-2 units): P = exp2(x - ref).
-    // The reference is the maximum of the row's first item; a later item whose
-    // exponentials sum to more than kMaxItemSum raises it to its own maximum
-    // (when that lies more than 8 above), O (all earlier P V complete) and the
-    // row sums being rescaled exactly.  So P stays below 2^24 (an |V| of 2^100 does
-    // not overflow O), and a maximum
-    // over the item's columns is not part of an ordinary step.
+    // Where some row's maximum over the item lies more than kRefSlack above its
+    // reference, every row of the warp that lies below its own maximum takes that
+    // as its reference, and the row sums and O are rescaled: O after the item's
+    // exponentials, when the P V before it is long complete.  So P stays below
+    // 2^kRefSlack.
+    // Only the element the reference comes from is exact in bf16, so a reference
+    // nearer to the maximum makes O's error smaller; at 6 the error against 64
+    // bits is that of whole-tile items raised past 2^8.  12 layers of 8 x 1024
+    // and 4 x 4096 tokens (w = 256) and a layer of 2 x 3000 (w = 512): 283, 1368
+    // and 86 us; at 8 with errors 1 to 2 % larger 281, 1350 and 85.5; with no
+    // maximum unless the exponentials of an item sum to 2^24, 3 to 4 % larger,
+    // 279, 1329 and 84; the same past 2^8 by a second evaluation of the item
+    // and O rescaled before it, 314, 1628 and 99.
     // lsum: the row sum of the exponentials (fp32), which gives the row's LSE
     // for the column sums; osum: the sum of the same values rounded to the
     // bf16 that P V multiplies, which normalises O (so that O is a weighted
     // mean of V rows whatever the rounding of P)
     float m_ref = i < n ? -INFINITY : 0.f, lsum = 0.f, osum = 0.f;
-    auto raise_to = [&](float tmax, bool may, bool have_o) {
-      const bool raise = may && tmax > m_ref + 8.f;
-      if (__any_sync(0xffffffffu, raise)) {
-        float f = 1.f;
-        if (raise) {
-          f = (m_ref == -INFINITY) ? 0.f : ex2(m_ref - tmax);
-          m_ref = tmax;
-          lsum *= f;
-          osum *= f;
-        }
-        if (have_o && __any_sync(0xffffffffu, f != 1.f)) {
-          // the item before this one: its P V, hence every earlier one
-          const int pb = buf == 0 ? kBufs - 1 : buf - 1;
-          ok = ok && warp_wait_poll(&sm.bar_pv[pb], (buf == 0 ? use - 1 : use) & 1, abort_flag);
-          tc_fence_after();
-#pragma unroll 1
-          for (int c = 0; c < 64; c += 16) {
-            float o[16];
-            tmem_ld16(tO + c, o);
-            tmem_ld_wait();
-#pragma unroll
-            for (int k = 0; k < 16; ++k) o[k] *= f;
-            tmem_st16(tO + c, reinterpret_cast<const uint32_t*>(o));
-            tmem_st_wait();   // o is reused
-          }
-        }
+    // raise_to returns the factor that the row's O takes (see rescale)
+    auto raise_to = [&](float tmax) {
+      float f = 1.f;
+      if (__any_sync(0xffffffffu, i < n && tmax > m_ref + kRefSlack) && i < n && tmax > m_ref) {
+        f = m_ref == -INFINITY ? 0.f : ex2(m_ref - tmax);
+        m_ref = tmax;
+        lsum *= f;
+        osum *= f;
       }
+      return f;
+    };
+    auto rescale = [&](float f) {
+      if (!__any_sync(0xffffffffu, f != 1.f)) return;
+      // the item before this one: its P V, hence every earlier one
+      const int pb = buf == 0 ? kBufs - 1 : buf - 1;
+      ok = ok && warp_wait_poll(&sm.bar_pv[pb], (buf == 0 ? use - 1 : use) & 1, abort_flag);
+      tc_fence_after();
+#pragma unroll 1
+      for (int c = 0; c < 64; c += 32) {
+        float o[32];
+        tmem_ld32(tO + c, o);
+        tmem_ld_wait();
+#pragma unroll
+        for (int k = 0; k < 32; ++k) o[k] *= f;
+        tmem_st32(tO + c, o);
+      }
+      tmem_st_wait();
     };
 #pragma unroll 1
     for (int it = 0; it < nrow - (glob ? 1 : 0); ++it) {
@@ -583,62 +590,47 @@ __global__ void __launch_bounds__(kRowsThreads, 2)
       if (kind0 == 1) mask_range(x, lo - j0, hi - j0);
       if (kind1 == 1) mask_range(x + 32, lo - j0 - 32, hi - j0 - 32);
       uint32_t pk[kHalf / 2];
-      float ls, os;
-      // at most twice: again with a raised reference for the rows whose sums
-      // came out too large under the old one (the maximum is looked for only
-      // then, and while a row of the warp has no reference yet; every row
-      // decides by its own values)
-      bool may = m_ref == -INFINITY;
-#pragma unroll 1
-      for (bool again = false;; again = true) {
-        if (__any_sync(0xffffffffu, may)) {
-          float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+      float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-          for (int ch = 0; ch < 2; ++ch)
-            if (ch ? kind1 : kind0)
+      for (int ch = 0; ch < 2; ++ch)
+        if (ch ? kind1 : kind0)
 #pragma unroll
-              for (int k = 32 * ch; k < 32 * ch + 32; k += 8)
+          for (int k = 32 * ch; k < 32 * ch + 32; k += 8)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) mx[e] = fmax3(mx[e], x[k + 2 * e], x[k + 2 * e + 1]);
-          raise_to(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * kLogitScale2, may,
-                   it > 0);
-        }
-        const float nref = m_ref == -INFINITY ? 0.f : -m_ref;
-        const uint64_t n2 = f2_pack(nref, nref);
-        uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
-        float sq[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int e = 0; e < 4; ++e) mx[e] = fmax3(mx[e], x[k + 2 * e], x[k + 2 * e + 1]);
+      const float f = raise_to(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * kLogitScale2);
+      const float nref = m_ref == -INFINITY ? 0.f : -m_ref;
+      const uint64_t n2 = f2_pack(nref, nref);
+      uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
+      float sq[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int ch = 0; ch < 2; ++ch) {
-          if (ch ? kind1 : kind0) {
+      for (int ch = 0; ch < 2; ++ch) {
+        if (ch ? kind1 : kind0) {
 #pragma unroll
-            for (int k = 32 * ch; k < 32 * ch + 32; k += 2) {
-              float u, e;
-              f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, n2), u, e);
-              u = ex2(u);
-              e = ex2(e);
-              const uint32_t q = pack_bf16x2(u, e);
-              pk[k >> 1] = q;
-              if (k & 2) s2b = f2_add(s2b, f2_pack(u, e));
-              else s2a = f2_add(s2a, f2_pack(u, e));
-              const int c = (k >> 1) & 1;
-              sq[2 * c] = add_bf16_lo(sq[2 * c], q);
-              sq[2 * c + 1] = add_bf16_hi(sq[2 * c + 1], q);
-            }
-          } else {
-#pragma unroll
-            for (int k = 16 * ch; k < 16 * ch + 16; ++k) pk[k] = 0u;
+          for (int k = 32 * ch; k < 32 * ch + 32; k += 2) {
+            float u, e;
+            f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, n2), u, e);
+            u = ex2(u);
+            e = ex2(e);
+            const uint32_t q = pack_bf16x2(u, e);
+            pk[k >> 1] = q;
+            if (k & 2) s2b = f2_add(s2b, f2_pack(u, e));
+            else s2a = f2_add(s2a, f2_pack(u, e));
+            const int c = (k >> 1) & 1;
+            sq[2 * c] = add_bf16_lo(sq[2 * c], q);
+            sq[2 * c + 1] = add_bf16_hi(sq[2 * c + 1], q);
           }
+        } else {
+#pragma unroll
+          for (int k = 16 * ch; k < 16 * ch + 16; ++k) pk[k] = 0u;
         }
-        float sa, sb, sc2, sd;
-        f2_unpack(s2a, sa, sb);
-        f2_unpack(s2b, sc2, sd);
-        ls = (sa + sb) + (sc2 + sd);
-        os = (sq[0] + sq[1]) + (sq[2] + sq[3]);
-        may = i < n && !(ls <= kMaxItemSum);
-        if (again || !__any_sync(0xffffffffu, may)) break;
       }
-      lsum += ls;
-      osum += os;
+      float sa, sb, sc2, sd;
+      f2_unpack(s2a, sa, sb);
+      f2_unpack(s2b, sc2, sd);
+      lsum += (sa + sb) + (sc2 + sd);
+      osum += (sq[0] + sq[1]) + (sq[2] + sq[3]);
+      if (it > 0) rescale(f);
       tmem_st16(tS, pk);
       tmem_st16(tS + 16, pk + 16);
       tmem_st_wait();
@@ -666,7 +658,7 @@ __global__ void __launch_bounds__(kRowsThreads, 2)
           load4(g0, x);
           mx = fmaxf(fmax3(mx, x[0], x[1]), fmaxf(x[2], x[3]));
         }
-        raise_to(mx, true, true);
+        rescale(raise_to(mx));
         const float nref = m_ref == -INFINITY ? 0.f : -m_ref;
 #pragma unroll 1
         for (int g0 = 0; g0 < kMaxGlobal; g0 += 4) {

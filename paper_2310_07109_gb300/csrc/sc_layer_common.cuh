@@ -1,6 +1,6 @@
 // sc_layer_common.cuh -- device helpers shared by the per-layer attention
-// kernels (the paired rows kernel, the single-pass band kernel and the cols
-// kernel): the resolved per-layer fields, TMA loads of 128-row tiles and of
+// kernels (rows, scores, the single-pass band kernel and the cols kernel behind
+// it): the resolved per-layer fields, TMA loads of 128-row tiles and of
 // the global rows, the QK^T / PV tcgen05 issue sequences, bounded waits, warp
 // reductions.
 #pragma once
