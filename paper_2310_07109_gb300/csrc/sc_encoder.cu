@@ -638,7 +638,9 @@ cudaError_t launch_gemm(const GemmParams& p, cudaStream_t st) {
   const long long tiles = static_cast<long long>(p.B) * ((p.L + kTile - 1) / kTile) *
                           ((p.N + least - 1) / least);
   const unsigned grid = static_cast<unsigned>(tiles < sms ? tiles : sms);
-  return launch_pdl(p.res == nullptr && !p.out_f32 ? sc_gemm_kernel<true> : sc_gemm_kernel<false>, dim3(grid), dim3(kGemmThreads), kGemmDyn, st, p);
+  const bool plain = p.res == nullptr && !p.out_f32;
+  return launch_pdl(plain ? sc_gemm_kernel<true> : sc_gemm_kernel<false>, dim3(grid),
+                    dim3(kGemmThreads), kGemmDyn, st, p);
 }
 
 cudaError_t launch_row_gather(const RowGatherParams& p, cudaStream_t st) {

@@ -58,6 +58,14 @@ constexpr uint32_t kTailColBytes = 2 * kTailMaxHeads * kTailMax * 4;
 constexpr uint32_t kTailDyn = 3 * kTailOpBytes + kTailStageBytes + kTailColBytes + 1024;
 static_assert(kTailDyn > 233472 / 2, "the tail kernel must occupy an SM alone");
 
+// Windows of kWideWindow and more have an instance whose layers of more than
+// kWideFrom tokens take 64 columns at a time, unrolled, without a test for empty
+// chunks (there are next to none): 12 layers, 8 sequences of 384 tokens, nothing
+// pruned, all pairs allowed 297 us instead of 321.  Smaller layers, and narrow
+// windows, lose by the longer code (24 x 128, w = 64: 218 instead of 210, even
+// where the wide loops are in the kernel but not taken): hence the instance.
+constexpr int kWideWindow = 192, kWideFrom = 192;
+
 struct TailSmem {
   uint64_t bar_cols[2];               // every head's column sums of a layer (by parity) are here
   uint64_t bar_sfull[2], bar_sfree[2], bar_pready[2], bar_odone[2], bar_stfull[2], bar_fin[2];
@@ -128,6 +136,7 @@ __device__ __forceinline__ void apply_mask(float* x, uint32_t m) {
 
 __device__ __forceinline__ int round16(int x) { return (x + 15) & ~15; }
 
+template <bool kWide>
 __global__ void __launch_bounds__(kTailThreads, 1)
     sc_tail_kernel(const __grid_constant__ TailParams p) {
   // the successor may start once every CTA is past its own grid wait, so it
@@ -277,6 +286,7 @@ __global__ void __launch_bounds__(kTailThreads, 1)
       }
     };
 
+    const bool wide = kWide && n > kWideFrom;
     if (warp >= 8) {
       // ------------------------------------------------------- MMA issue
       const int X = warp - 8;
@@ -350,6 +360,29 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         me.all = w >= n - 1 || ((sm.gbits[cur][i >> 5] >> (i & 31)) & 1u);
         return me;
       };
+      // half 1 against the reference of half 0
+      auto raise_half = [&](float mx, float& ref, float& lsum, float& osum) {
+        const bool raise = mx > ref + 8.f;
+        if (__any_sync(0xffffffffu, raise)) {
+          float f = 1.f;
+          if (raise) {
+            f = ref == -INFINITY ? 0.f : ex2(ref - mx);
+            ref = mx;
+            lsum *= f;
+            osum *= f;
+          }
+#pragma unroll 1
+          for (int c = 0; c < 64; c += 32) {
+            float o[32];
+            tmem_ld32(tO + c, o);
+            tmem_ld_wait();
+#pragma unroll
+            for (int k = 0; k < 32; ++k) o[k] *= f;
+            tmem_st32(tO + c, o);
+            tmem_st_wait();   // o is reused
+          }
+        }
+      };
       // Softmax of half kh (S in tensor memory), 32 keys at a time, in two passes:
       // the row's maximum over the half, then P = exp2(S - ref), written as bf16
       // pairs over the first half of the columns (each chunk's pairs land on
@@ -373,13 +406,15 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         uint32_t some = 0u;   // chunks inside some row's window (warp-uniform)
 #pragma unroll 1
         for (int q = 0; q < chunks; ++q) {
-          const uint32_t in = partner_mask(me, sm, cur, 8 * kh + q, n);
-          if (!__any_sync(0xffffffffu, in != 0u)) continue;
-          some |= 1u << q;
           float x[32];
           tmem_ld32(tR + 32 * q, x);
+          const uint32_t in = partner_mask(me, sm, cur, 8 * kh + q, n);
+          const bool any = __any_sync(0xffffffffu, in != 0u);
+          const bool full = __all_sync(0xffffffffu, in == 0xffffffffu);
           tmem_ld_wait();
-          if (!__all_sync(0xffffffffu, in == 0xffffffffu)) {
+          if (!any) continue;
+          some |= 1u << q;
+          if (!full) {
 #pragma unroll
             for (int k = 0; k < 32; ++k) x[k] = ((in >> k) & 1u) ? x[k] : -INFINITY;
             tmem_st32(tR + 32 * q, x);   // masked: the second pass takes it as it is
@@ -397,29 +432,12 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         if (kh == 0) {
           ref = mx;
         } else {
-          const bool raise = mx > ref + 8.f;
-          if (__any_sync(0xffffffffu, raise)) {
-            float f = 1.f;
-            if (raise) {
-              f = ref == -INFINITY ? 0.f : ex2(ref - mx);
-              ref = mx;
-              lsum *= f;
-              osum *= f;
-            }
-#pragma unroll 1
-            for (int c = 0; c < 64; c += 8) {
-              float o[8];
-              tmem_ld8(tO + c, o);
-              tmem_ld_wait();
-#pragma unroll
-              for (int k = 0; k < 8; ++k) o[k] *= f;
-              tmem_st8(tO + c, reinterpret_cast<const uint32_t*>(o));
-              tmem_st_wait();   // o is reused
-            }
-          }
+          raise_half(mx, ref, lsum, osum);
         }
         const float nref = ref == -INFINITY ? 0.f : -ref;
         const uint64_t n2 = f2_pack(nref, nref);
+        uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
+        float sq[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
         for (int q = 0; q < chunks; ++q) {
           uint32_t pk[16];
@@ -430,8 +448,6 @@ __global__ void __launch_bounds__(kTailThreads, 1)
             float x[32];
             tmem_ld32(tR + 32 * q, x);
             tmem_ld_wait();
-            uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
-            float sq[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int k = 0; k < 32; k += 2) {
               float u, v;
@@ -446,15 +462,77 @@ __global__ void __launch_bounds__(kTailThreads, 1)
               sq[2 * c] = add_bf16_lo(sq[2 * c], b2);
               sq[2 * c + 1] = add_bf16_hi(sq[2 * c + 1], b2);
             }
-            float ea, eb, ec, ed;
-            f2_unpack(s2a, ea, eb);
-            f2_unpack(s2b, ec, ed);
-            lsum += (ea + eb) + (ec + ed);
-            osum += (sq[0] + sq[1]) + (sq[2] + sq[3]);
           }
           tmem_st16(tR + 16 * q, pk);
         }
+        float ea, eb, ec, ed;
+        f2_unpack(s2a, ea, eb);
+        f2_unpack(s2b, ec, ed);
+        lsum += (ea + eb) + (ec + ed);
+        osum += (sq[0] + sq[1]) + (sq[2] + sq[3]);
         tmem_st_wait();
+      };
+      // The same for layers with wide windows: 64 columns at a time, no chunk is
+      // empty, masks where a warp needs them.  Row maximum over the keys of half kh.
+      auto half_max = [&](const Partners& me, int kh, float mx) {
+        const int nh = min(256, n - 256 * kh);
+        for (int q2 = 0; q2 < (nh + 63) >> 6; ++q2) {
+          float x[64];
+          tmem_ld32(tR + 64 * q2, x);
+          tmem_ld32(tR + 64 * q2 + 32, x + 32);
+          tmem_ld_wait();
+#pragma unroll
+          for (int hq = 0; hq < 2; ++hq) {
+            apply_mask(x + 32 * hq, partner_mask(me, sm, cur, 8 * kh + 2 * q2 + hq, n));
+#pragma unroll
+            for (int k = 0; k < 32; k += 2) mx = fmax3(mx, x[32 * hq + k], x[32 * hq + k + 1]);
+          }
+        }
+        return mx;
+      };
+      // P of half kh against the reference -nmc; returns the sum of the
+      // exponentials and adds that of their bf16 values to *osum.
+      auto half_exp = [&](const Partners& me, int kh, float nmc, float* osum) {
+        const int nh = min(256, n - 256 * kh);
+        const uint64_t n2 = f2_pack(nmc, nmc);
+        uint64_t s2a = f2_pack(0.f, 0.f), s2b = s2a;
+        float la = 0.f, lb = 0.f, lc = 0.f, ld = 0.f;
+        for (int q2 = 0; q2 < (nh + 63) >> 6; ++q2) {
+          float x[64];
+          tmem_ld32(tR + 64 * q2, x);
+          tmem_ld32(tR + 64 * q2 + 32, x + 32);
+          tmem_ld_wait();
+#pragma unroll
+          for (int hq = 0; hq < 2; ++hq) {
+            float* xh = x + 32 * hq;
+            apply_mask(xh, partner_mask(me, sm, cur, 8 * kh + 2 * q2 + hq, n));
+            uint32_t pk[16];
+#pragma unroll
+            for (int k = 0; k < 32; k += 2) {
+              float u, v;
+              f2_unpack(f2_fma(f2_pack(xh[k], xh[k + 1]), c2, n2), u, v);
+              u = ex2(u);
+              v = ex2(v);
+              if (k & 2) s2b = f2_add(s2b, f2_pack(u, v));
+              else s2a = f2_add(s2a, f2_pack(u, v));
+              pk[k >> 1] = pack_bf16x2(u, v);
+              if (k & 2) {
+                lc = add_bf16_lo(lc, pk[k >> 1]);
+                ld = add_bf16_hi(ld, pk[k >> 1]);
+              } else {
+                la = add_bf16_lo(la, pk[k >> 1]);
+                lb = add_bf16_hi(lb, pk[k >> 1]);
+              }
+            }
+            tmem_st16(tR + 32 * q2 + 16 * hq, pk);
+          }
+        }
+        tmem_st_wait();
+        *osum += (la + lb) + (lc + ld);
+        float ea, eb, ec, ed;
+        f2_unpack(s2a, ea, eb);
+        f2_unpack(s2b, ec, ed);
+        return (ea + eb) + (ec + ed);
       };
       auto release = [&]() {   // the warpgroup's columns are read
         tc_fence_before();
@@ -471,18 +549,34 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         if (!(ok = tail_wait(&sm.bar_sfull[X], (n_sfull++) & 1, abort_flag))) break;
         tc_fence_after();
         float ref = -INFINITY, lsum = 0.f, osum = 0.f;
+        if (!wide) {
 #pragma unroll 1
-        for (int kh = 0; kh < nkh; ++kh) {
-          if (kh > 0) {
-            // half 1 (at most 128 keys; its S lands on P of half 0 after that
-            // half's P V, so O of half 0 is complete once S is)
+          for (int kh = 0; kh < nkh; ++kh) {
+            if (kh > 0) {
+              // half 1 (at most 128 keys; its S lands on P of half 0 after that
+              // half's P V, so O of half 0 is complete once S is)
+              if (!(ok = tail_wait(&sm.bar_sfull[X], (n_sfull++) & 1, abort_flag))) break;
+              if (!(ok = tail_wait(&sm.bar_odone[X], (n_odone++) & 1, abort_flag))) break;
+              tc_fence_after();
+            }
+            half_softmax(me, kh, ref, lsum, osum);
+            tc_fence_before();
+            warp_arrive(&sm.bar_pready[X]);
+          }
+        } else {
+          ref = half_max(me, 0, -INFINITY) * kLogitScale2;
+          lsum = half_exp(me, 0, ref == -INFINITY ? 0.f : -ref, &osum);
+          tc_fence_before();
+          warp_arrive(&sm.bar_pready[X]);
+          if (nkh > 1) {
             if (!(ok = tail_wait(&sm.bar_sfull[X], (n_sfull++) & 1, abort_flag))) break;
             if (!(ok = tail_wait(&sm.bar_odone[X], (n_odone++) & 1, abort_flag))) break;
             tc_fence_after();
+            raise_half(half_max(me, 1, -INFINITY) * kLogitScale2, ref, lsum, osum);
+            lsum += half_exp(me, 1, ref == -INFINITY ? 0.f : -ref, &osum);
+            tc_fence_before();
+            warp_arrive(&sm.bar_pready[X]);
           }
-          half_softmax(me, kh, ref, lsum, osum);
-          tc_fence_before();
-          warp_arrive(&sm.bar_pready[X]);
         }
         if (!ok) break;
         // rows' -LSE; a valid row attends to itself, so its reference is finite
@@ -524,24 +618,50 @@ __global__ void __launch_bounds__(kTailThreads, 1)
           if (!(ok = tail_wait(&sm.bar_stfull[X], (n_stfull++) & 1, abort_flag))) break;
           tc_fence_after();
           const int chunks = (min(256, n - 256 * qh) + 31) >> 5;
+          if (!wide) {
 #pragma unroll 1
-          for (int q = 0; q < chunks; ++q) {
-            const int qa = 8 * qh + q;   // chunk of query rows
-            const uint32_t in = partner_mask(me, sm, cur, qa, n);
-            if (!__any_sync(0xffffffffu, in != 0u)) continue;   // outside every window
-            float x[32];
-            tmem_ld32(tST + 32 * q, x);
-            tmem_ld_wait();
-            apply_mask(x, in);
-            const float* lw = sm.nlse + 32 * qa;
+            for (int q = 0; q < chunks; ++q) {
+              const int qa = 8 * qh + q;   // chunk of query rows
+              float x[32];
+              tmem_ld32(tST + 32 * q, x);
+              const uint32_t in = partner_mask(me, sm, cur, qa, n);
+              const bool any = __any_sync(0xffffffffu, in != 0u);
+              tmem_ld_wait();
+              if (!any) continue;   // outside every window
+              apply_mask(x, in);
+              const float* lw = sm.nlse + 32 * qa;
 #pragma unroll
-            for (int k = 0; k < 32; k += 4) {
-              const float4 l4 = *reinterpret_cast<const float4*>(lw + k);
-              float e0, e1, e2, e3;
-              f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, f2_pack(l4.x, l4.y)), e0, e1);
-              f2_unpack(f2_fma(f2_pack(x[k + 2], x[k + 3]), c2, f2_pack(l4.z, l4.w)), e2, e3);
-              a2a = f2_add(a2a, f2_pack(ex2(e0), ex2(e1)));
-              a2b = f2_add(a2b, f2_pack(ex2(e2), ex2(e3)));
+              for (int k = 0; k < 32; k += 4) {
+                const float4 l4 = *reinterpret_cast<const float4*>(lw + k);
+                float e0, e1, e2, e3;
+                f2_unpack(f2_fma(f2_pack(x[k], x[k + 1]), c2, f2_pack(l4.x, l4.y)), e0, e1);
+                f2_unpack(f2_fma(f2_pack(x[k + 2], x[k + 3]), c2, f2_pack(l4.z, l4.w)), e2, e3);
+                a2a = f2_add(a2a, f2_pack(ex2(e0), ex2(e1)));
+                a2b = f2_add(a2b, f2_pack(ex2(e2), ex2(e3)));
+              }
+            }
+          } else {
+            for (int q2 = 0; q2 < (chunks + 1) >> 1; ++q2) {
+              float x[64];
+              tmem_ld32(tST + 64 * q2, x);
+              tmem_ld32(tST + 64 * q2 + 32, x + 32);
+              tmem_ld_wait();
+#pragma unroll
+              for (int hq = 0; hq < 2; ++hq) {
+                const int qa = 8 * qh + 2 * q2 + hq;   // chunk of query rows
+                float* xh = x + 32 * hq;
+                apply_mask(xh, partner_mask(me, sm, cur, qa, n));
+                const float* lw = sm.nlse + 32 * qa;
+#pragma unroll
+                for (int k = 0; k < 32; k += 4) {
+                  const float4 l4 = *reinterpret_cast<const float4*>(lw + k);
+                  float e0, e1, e2, e3;
+                  f2_unpack(f2_fma(f2_pack(xh[k], xh[k + 1]), c2, f2_pack(l4.x, l4.y)), e0, e1);
+                  f2_unpack(f2_fma(f2_pack(xh[k + 2], xh[k + 3]), c2, f2_pack(l4.z, l4.w)), e2, e3);
+                  a2a = f2_add(a2a, f2_pack(ex2(e0), ex2(e1)));
+                  a2b = f2_add(a2b, f2_pack(ex2(e2), ex2(e3)));
+                }
+              }
             }
           }
           if (nq > 1) release();
@@ -570,20 +690,22 @@ __global__ void __launch_bounds__(kTailThreads, 1)
       float sj[2] = {0.f, 0.f};
       const float inv_hn = static_cast<float>(H * n);
       __all_sync(0xffffffffu, mbar_wait_cluster(&sm.bar_cols[par], (it >> 1) & 1, abort_flag));
-#pragma unroll
-      for (int rd = 0; rd < 2; ++rd) {
+#pragma unroll 1
+      for (int rd = 0; rd < rounds; ++rd) {
         const int j = tid + 256 * rd;
-        if (rd < rounds && j < n) {
+        float a = 0.f;
+        if (j < n) {
           const float* cj = colall + par * kTailMaxHeads * kTailMax + j;
           float v[kTailMaxHeads];
 #pragma unroll
           for (int hh = 0; hh < kTailMaxHeads; ++hh) v[hh] = hh < H ? cj[hh * kTailMax] : 0.f;
-          float a = 0.f;
 #pragma unroll
           for (int hh = 0; hh < kTailMaxHeads; ++hh) a += v[hh];   // (zeros past H)
-          sj[rd] = a / inv_hn;
-          if (h == 0) out_scores[(static_cast<size_t>(l) * B + b) * L + j] = sj[rd];
+          a /= inv_hn;
+          if (h == 0) out_scores[(static_cast<size_t>(l) * B + b) * L + j] = a;
         }
+        if (rd == 0) sj[0] = a;
+        else sj[1] = a;
       }
       // keep flags: the threshold (relative or absolute), or the top-ratio cut
       // over the n scores (every CTA of the cluster finds the same cut)
@@ -679,10 +801,14 @@ __global__ void __launch_bounds__(kTailThreads, 1)
 // launch helpers used by the C ABI
 // ---------------------------------------------------------------------------
 cudaError_t configure_tail() {
-  cudaError_t e = cudaFuncSetAttribute(sc_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(kTailDyn));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(sc_tail_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaError_t e = cudaSuccess;
+  for (auto kernel : {sc_tail_kernel<false>, sc_tail_kernel<true>}) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               static_cast<int>(kTailDyn));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  }
   return e;
 }
 
@@ -708,7 +834,8 @@ cudaError_t tail_max_clusters(int H, int* out) {
   if (H < 1 || H > kTailMaxHeads) return cudaSuccess;
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = tail_config(1, H, nullptr, attr);
-  return cudaOccupancyMaxActiveClusters(out, sc_tail_kernel, &cfg);
+  // (both instances: the shared memory allows one CTA an SM)
+  return cudaOccupancyMaxActiveClusters(out, sc_tail_kernel<true>, &cfg);
 }
 
 cudaError_t launch_tail(const TailParams& p, cudaStream_t st) {
@@ -719,7 +846,7 @@ cudaError_t launch_tail(const TailParams& p, cudaStream_t st) {
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, sc_tail_kernel, p);
+  return cudaLaunchKernelEx(&cfg, p.w >= kWideWindow ? sc_tail_kernel<true> : sc_tail_kernel<false>, p);
 }
 
 }  // namespace sc
