@@ -88,9 +88,9 @@ constexpr uint32_t kPgBlock = 2 * 1024;
 // 78 KB of code instead of 55 KB the kernel missed the instruction caches and
 // took 14% longer.
 // Layer 0 of 2 x 4096 tokens (w 256, 12 heads, 9 global tokens), rows and scores
-// together: 81 us, against 89 us for pairs of query tiles in one CTA per SM
-// with whole-tile items and a tensor-core scores kernel; 4 x 4096: 113 against
-// 144 us; 3 x 1000 at w 64: 25 against 35 us.
+// together: 80 us, against 89 us for pairs of query tiles in one CTA per SM
+// with whole-tile items and a tensor-core scores kernel; 4 x 4096, one global
+// token: 117 against 145 us; 8 x 1024 at w 64: 45 against 71 us.
 constexpr int kRowsThreads = 256;
 constexpr int kKSlots = 3, kVSlots = 2;          // 16 KB operand slots
 constexpr int kRowsSlots = kKSlots + kVSlots;    // K tiles 0..2, V tiles 3..4
@@ -1337,7 +1337,12 @@ __global__ void __launch_bounds__(kExportThreads)
   for (int it = blockIdx.x; it < items; it += gridDim.x) {
     const int ch = it % nch, lb = it / nch;
     const int b = lb % e.B, l = lb / e.B;
-    if (e.part != 0 && (e.part == 1) != (l < __ldcg(e.tail_from + b))) continue;
+    if (e.part != 0) {
+      // a sequence that first gets short after the last layer has no layer in the
+      // cluster kernel: its last slot is the per-layer kernels' too
+      const int from = __ldcg(e.tail_from + b);
+      if ((e.part == 1) != (l < from || from >= e.n_layers)) continue;
+    }
     const size_t li = static_cast<size_t>(l) * e.B + b;
     const int n = __ldcg(e.len + li);
     if (ch == 0 && threadIdx.x == 0) e.hlen[li] = n;
