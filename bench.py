@@ -605,15 +605,17 @@ def run_native(args, wl):
     t_roof = sum(max(Bb / bw, Ff / fl) for Bb, Ff in work)
     t_meas = (float((rows_ms + cols_ms).sum()) + tail_ms) * 1e-3
     # the dominant unit: the per-layer kernel pair of the full-length layer 0
-    # (rows + cols, one launch each); when every sequence starts in the cluster
+    # (rows + scores, one launch each); when every sequence starts in the cluster
     # kernel, that kernel over all layers
     t_l0 = pair_ms * 1e-3
+    pair_kernels = (("sc_rows_kernel", "sc_scores_kernel") if args.rows_kernel == "two-pass"
+                    else ("sc_band_kernel", "sc_cols_kernel"))
     if rows_ms[0] + cols_ms[0] > 1e-6:
         unit_bytes, unit_flops, unit_t = work[0][0], work[0][1], t_l0
-        unit_kernels = ["sc_rows_kernel", "sc_cols_kernel"]
-        unit_desc = ("sc_rows_kernel + sc_scores_kernel of layer 0 (one launch each, chained "
+        unit_kernels = list(pair_kernels)
+        unit_desc = ("%s + %s of layer 0 (one launch each, chained "
                      "as in the timed step; B=%d sequences of %d tokens)"
-                     % (wl.B, int(lens[0].max())))
+                     % (pair_kernels + (wl.B, int(lens[0].max()))))
     else:
         unit_bytes = sum(Bb for Bb, _ in work)
         unit_flops = sum(Ff for _, Ff in work)
@@ -635,15 +637,14 @@ def run_native(args, wl):
                         "per_unit": "6152 B per token-layer; 3072 flop per allowed (query, "
                                     "key) pair (all heads, QK^T and PV)"},
         "launch_ms": unit_t * 1e3,
-        "serialised_ms": (float(rows_ms[0] + cols_ms[0]) if unit_kernels[0] == "sc_rows_kernel"
+        "serialised_ms": (float(rows_ms[0] + cols_ms[0]) if unit_kernels[0] == pair_kernels[0]
                           else unit_t * 1e3),
         "traffic_note": traffic_note,
         "stack_frac": t_roof / t_meas,
         "stack_scope": "sum over layers of max(F_l/peak_bf16, B_l/peak_hbm) over the measured "
-                       "time of sc_rows_kernel + sc_cols_kernel (per-layer layers) and "
-                       "sc_tail_kernel",
-        "kernel_ms_per_step": {"sc_rows_kernel": float(rows_ms.sum()),
-                               "sc_cols_kernel": float(cols_ms.sum()),
+                       "time of %s + %s (per-layer layers) and sc_tail_kernel" % pair_kernels,
+        "kernel_ms_per_step": {pair_kernels[0]: float(rows_ms.sum()),
+                               pair_kernels[1]: float(cols_ms.sum()),
                                "sc_gather_kernel": float(gath_ms.sum()),
                                "sc_prep_kernel": prep_ms,
                                "sc_tail_kernel": tail_ms},
