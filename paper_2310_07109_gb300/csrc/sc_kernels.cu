@@ -347,6 +347,11 @@ __global__ void __launch_bounds__(kRowsThreads, 2)
             const bool g = it >= nblk;
             const int slot = kKSlots + (t & 1);
             if (!g && !(ok = warp_wait_poll(&sm.full[slot], (t / kVSlots) & 1, abort_flag))) break;
+            if (!g && (kb + 1) * kHalf > n) {   // (the last block)
+              zero_rows(Slots + slot * kTileBytes, n - (klo + t) * kTile, kHalf * ((kb & 1) + 1),
+                        lane, 32);
+              __syncwarp();
+            }
             tc_fence_after();
             const uint32_t v_d = g ? vg_d : slot_d + slot * kTileD + (kb & 1) * kHalfD;
             if (elect_one()) {
@@ -469,6 +474,10 @@ __global__ void __launch_bounds__(kRowsThreads, 2)
       if (warp == 6) {
         ok = ok && warp_wait_poll(&sm.bar_vd, 0, abort_flag);
         if (ok) {
+          if (q0 + kTile > n) {
+            zero_rows(Slots + vd_slot * kTileBytes, n - q0, kTile, lane, 32);
+            __syncwarp();
+          }
           tc_fence_after();   // O is out: its columns take the product
           if (elect_one()) {
             mma_pv(tm + kColO, smem_u32(Pg) - kPgRow0 * 128, kPgBlock,

@@ -106,6 +106,18 @@ __device__ __forceinline__ void load_tile(const TensorMaps& m, int t, const RowS
   tma_load_3d(dst, &m.tile[rs.s][t], 0, h, static_cast<int>(rs.tok_b + c0), bar);
 }
 
+// Rows from .. to - 1 of an operand tile in shared memory become zero, for the
+// matrix products that follow (the caller is a whole warp, or one thread as lane 0
+// of 1, and the tile has landed).  P V multiplies whole 16-row blocks: rows past the
+// sequence's end have P = 0, but 0 x Inf and 0 x NaN are NaN, and what lies there is
+// the caller's padding, another sequence or an earlier use of the workspace.
+__device__ __forceinline__ void zero_rows(uint8_t* tile, int from, int to, int lane, int lanes) {
+#pragma unroll 1
+  for (int k = 8 * from + lane; k < 8 * to; k += lanes)
+    reinterpret_cast<uint4*>(tile)[k] = make_uint4(0u, 0u, 0u, 0u);
+  fence_proxy_async_smem();
+}
+
 // The 16 global rows (current indices gc[0..ng-1], the last repeated): lanes
 // 0..3 gather four rows each.
 __device__ __forceinline__ void load_globals(const TensorMaps& m, int t, const RowSource& rs, int h,
