@@ -438,8 +438,14 @@ __global__ void __launch_bounds__(kBandThreads, 1)
             // the first product overwrites O: the helpers have read the previous item's
             if (t == 0 && item_no > 0 && !mbar_wait(&sm.bar_ofree, (item_no - 1) & 1, abort_flag))
               return false;
+            int steps = kTile / 16;
+            const int left = x.n - (x.klo + t) * kTile;   // the tile's keys before the end
+            if (left < kTile) {
+              steps = (left + 15) / 16;
+              zero_rows(base + kOffV + vs * kTileBytes, left, 16 * steps, 0, 1);
+            }
             tc_fence_after();
-            mma_pv_ts(tm + kColO, tm + col_slot(t), v_a + vs * kTileBytes, kTile / 16, t > 0);
+            mma_pv_ts(tm + kColO, tm + col_slot(t), v_a + vs * kTileBytes, steps, t > 0);
             umma_commit(&sm.bar_vempty[vs]);
             umma_commit(&sm.bar_pvdone[t]);
             committed |= 1u << t;

@@ -966,9 +966,15 @@ __global__ void __launch_bounds__(kColsThreads, 2)
       if (ok && ngp)
         for (int X = 0; ok && X < nX; ++X) {
           if (!(ok = mbar_wait(&sm.bar_pg[X], 0, abort_flag))) break;
+          int steps = kTile / 16;
+          const int left = n - (2 * pr + X) * kTile;   // the tile's keys before the end
+          if (left < kTile) {
+            steps = (left + 15) / 16;
+            zero_rows(Vs + X * kTileBytes, left, 16 * steps, 0, 1);
+          }
           tc_fence_after();
           mma_pv(tm + 64 + 64 * X, smem_u32(Pg) + X * 2 * kPgBlock, kPgBlock, v_a + X * kTileBytes,
-                 kTile / 16, false);
+                 steps, false);
           umma_commit(&sm.bar_og[X]);
         }
       umma_commit(&sm.bar_fin);

@@ -50,6 +50,16 @@ def test_layer_rows_past_length(L, lens, w, gl, H):
     _check_layer_past_length(sc, L, lens, w, gl, H)
 
 
+@pytest.mark.parametrize("gl", [[], [0, 1, 70]], ids=["band", "globals"])
+def test_single_pass_layer_rows_past_length(gl):
+    import paper_2310_07109_gb300 as sc
+    sc.select_rows_kernel(sc.SC_ROWS_SINGLE_PASS)
+    try:
+        _check_layer_past_length(sc, 640, [577, 0, 640, 513], 64, gl, 4)
+    finally:
+        sc.select_rows_kernel(sc.SC_ROWS_TWO_PASS)
+
+
 STACKS = [
     wk.Workload("pruned_4x700", n_layers=4, B=2, L=700, H=4, w=64, n_extra_global=3,
                 ragged=(600, 690), seed=41),
