@@ -234,16 +234,19 @@ __global__ void __launch_bounds__(kTailThreads, 1)
     // ---- rows of the current tokens: 16-byte pieces, 128B-swizzled tiles
     {
       // thread tid copies 16-byte piece (tid & 7) of every 40th row, the
-      // same piece of Q, K and V from one address computation
+      // same piece of Q, K and V from one address computation.  Rows up to the end
+      // of the last 16-row block of P V become zero: they meet P = 0 there, but a
+      // NaN or infinity in the V that a pruned token left would still reach O
+      // (filled by the copies: separate stores took 0.14 us a layer).
       const size_t tok0 = (static_cast<size_t>(l) * B + b) * L;
       const int piece = tid & 7;
 #pragma unroll 2
-      for (int r = tid >> 3; r < n; r += kTailThreads / 8) {
-        const size_t off = ((tok0 + sm.pos[cur][r]) * H + h) * kHeadDim + 8 * piece;
+      for (int r = tid >> 3; r < round16(n); r += kTailThreads / 8) {
+        const size_t off = ((tok0 + sm.pos[cur][min(r, n - 1)]) * H + h) * kHeadDim + 8 * piece;
         const uint32_t so = sw128_offset(r, piece);
-        cp_async16(q_a + so, p.src[0] + off);
-        cp_async16(k_a + so, p.src[1] + off);
-        cp_async16(v_a + so, p.src[2] + off);
+        cp_async16(q_a + so, p.src[0] + off, r < n);
+        cp_async16(k_a + so, p.src[1] + off, r < n);
+        cp_async16(v_a + so, p.src[2] + off, r < n);
       }
       if (l + 1 < n_layers && !p.src_host) {
         // the next layer's tokens are a subset of the current ones

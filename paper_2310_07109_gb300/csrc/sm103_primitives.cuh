@@ -520,9 +520,12 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
 }
 
 // 16-byte global -> shared copy through the load/store path (no register
-// staging); completes at cp_async_wait_all().  Writes via the generic proxy.
-__device__ __forceinline__ void cp_async16(uint32_t saddr, const void* gptr) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(gptr) : "memory");
+// staging), or 16 zero bytes without reading gptr; completes at
+// cp_async_wait_all().  Writes via the generic proxy.
+__device__ __forceinline__ void cp_async16(uint32_t saddr, const void* gptr, bool copy) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(saddr), "l"(gptr),
+               "r"(copy ? 16 : 0)
+               : "memory");
 }
 
 __device__ __forceinline__ void cp_async_wait_all() {

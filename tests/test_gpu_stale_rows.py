@@ -1,11 +1,12 @@
 """Rows that hold no current token never reach a result: the operand tiles of the
 matrix products take whole 16-, 64- or 128-row blocks, so they contain rows past a
 sequence's length (the caller's padding, the next sequence's tokens, whatever the
-workspace held before).  Here those rows are NaN."""
+workspace held before, tokens that a layer pruned).  Here those rows are NaN."""
 import numpy as np
 import pytest
 import torch
 
+import oracle
 import workloads as wk
 from parity_utils import (bits_to_torch, check_o, check_scores, check_stack, layer_case,
                           resample_stack, torch_bf16_to_f64)
@@ -82,6 +83,30 @@ def test_stack_dirty_workspace_and_padding(wl, no_tail):
     assert sc.workspace_status(ws) == 0
     check_stack(wl, res, {"O": torch_bf16_to_f64(out["O"]), "scores": out["scores"].cpu().numpy(),
                           "pos": out["pos"].cpu().numpy(), "len": out["len"].cpu().numpy()})
+
+
+@pytest.mark.parametrize("w", [64, 230])
+@pytest.mark.parametrize("L,rho", [(200, 0.5), (380, 0.7)])
+def test_cluster_kernel_rows_of_pruned_tokens(L, rho, w):
+    """The first layer's V is NaN at the slots just past the second layer's length."""
+    import paper_2310_07109_gb300 as sc
+    wl = wk.Workload("stale", n_layers=2, B=2, L=L, H=4, w=w, n_extra_global=2, alpha_first=rho,
+                     alpha_last=1.0, keep_rule=oracle.KEEP_TOP_RATIO, seed=43)
+    inp, res, _ = resample_stack(wl)
+    n1 = int(res["len"][1, 0])
+    assert n1 % 16 != 0
+    inp["V"][0, :, n1:n1 + 16] = NAN
+    Q, K, V = (bits_to_torch(inp[k], "cuda") for k in ("Q", "K", "V"))
+    out = sc.stack_forward(Q, K, V, None, inp["global_pos"], wl.w, inp["alpha"],
+                           keep_rule=wl.keep_rule)
+    np.testing.assert_array_equal(out["len"].cpu().numpy(), res["len"])
+    pos, s, O = out["pos"].cpu().numpy(), out["scores"].cpu().numpy(), torch_bf16_to_f64(out["O"])
+    for b in range(wl.B):
+        np.testing.assert_array_equal(pos[1, b, :n1], res["pos"][1, b, :n1])
+        for l in range(2):
+            n = int(res["len"][l, b])
+            check_scores(s[l, b, :n], res["scores"][l, b, :n], f"layer {l} seq {b}")
+        check_o(O[1, b, :n1], res["O"][1, b, :n1], f"seq {b}")
 
 
 def test_encoder_layer_dirty_workspace():
