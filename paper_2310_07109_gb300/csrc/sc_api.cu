@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -457,6 +458,10 @@ int layer_forward_impl(const sc_layer_args* a, void* workspace, size_t ws_bytes,
 // Layers per turn of the device-driven loop: a turn costs about 7 us beside its
 // kernels, a layer that nothing needs about as much, so one such layer at most.
 constexpr int kLoopLayers = 2;
+// Layers of one conditional group of a padded stack under the top-ratio rule (see
+// stack_forward_impl): a group costs 7 to 13 us beside its kernels, a layer in it
+// that nothing needs 4 to 13 us (its empty grids grow with B L).
+constexpr int kGroupLayers = 6;
 
 // Which kernels a stack call launches: sequences with at most kTailMax tokens
 // left finish in the cluster kernel (when it can run with clusters of H CTAs);
@@ -598,10 +603,59 @@ static int stack_forward_impl(const sc_stack_args* a, void* workspace, size_t ws
   // every turn costs about 7 us beside its kernels (3 x 1000 tokens, nothing
   // pruned, 12 layers: 371 us with the loop, 286 without; 4 x 777, top ratio:
   // 428 and 381).
+  // With padding the bound holds for L and not for the true lengths, so there the
+  // layers run only where some sequence is longer than kTailMax: all of them in
+  // one IF node where nothing is pruned, in groups of kGroupLayers under the
+  // top-ratio rule.  12 layers, one after the other / two a turn of the loop / so:
+  // 4 x 4096 with at most 384 tokens, unpruned 492 / 355 / 334 us, top ratio 402 /
+  // 264 / 247; with at most 500 tokens, top ratio 471 / 411 / 416; 3 x 1000 with
+  // one of full length, unpruned 289 / 350 / 306; 4 x 2048 likewise, top ratio
+  // 597 / 685 / 618 (groups of 4: 631, one group: 603 but 497 with 500 tokens).
   bool dev_loop = false;
   int direct = a->n_layers;   // layers launched directly when there is no loop
+  int group = 0;              // ... in conditional groups of so many, unless 0
   cudaGraphConditionalHandle cond = 0;
   cudaStream_t side = nullptr;
+  // a condition of the graph being captured, false until a kernel sets it
+  auto new_condition = [&](cudaGraphConditionalHandle* h) -> int {
+    cudaGraph_t g = nullptr;
+    cudaStreamCaptureStatus cs;
+    if ((e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &g)) != cudaSuccess)
+      return fail_cuda("stream capture info", e);
+    e = cudaGraphConditionalHandleCreate(h, g, 0, cudaGraphCondAssignDefault);
+    return e == cudaSuccess ? SC_OK : fail_cuda("conditional handle", e);
+  };
+  // a WHILE or IF node after the work captured on st so far, whose body is what
+  // `body` launches on the side stream
+  auto add_conditional = [&](cudaGraphConditionalNodeType type, cudaGraphConditionalHandle h,
+                             const std::function<int()>& body) -> int {
+    cudaGraph_t g = nullptr;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t ndeps = 0;
+    cudaStreamCaptureStatus cs;
+    if ((e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, &deps, nullptr, &ndeps)) != cudaSuccess)
+      return fail_cuda("stream capture info", e);
+    cudaGraphNodeParams cp = {};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = h;
+    cp.conditional.type = type;
+    cp.conditional.size = 1;
+    cudaGraphNode_t node;
+    if ((e = cudaGraphAddNode(&node, g, deps, nullptr, ndeps, &cp)) != cudaSuccess)
+      return fail_cuda("add conditional node", e);
+    if ((e = cudaStreamBeginCaptureToGraph(side, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                           cudaStreamCaptureModeRelaxed)) != cudaSuccess)
+      return fail_cuda("capture conditional body", e);
+    const int brc = body();
+    cudaGraph_t done = nullptr;
+    e = cudaStreamEndCapture(side, &done);
+    if (brc != SC_OK) return brc;
+    if (e != cudaSuccess) return fail_cuda("end conditional body capture", e);
+    if ((e = cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1,
+                                                 cudaStreamSetCaptureDependencies)) != cudaSuccess)
+      return fail_cuda("capture dependencies", e);
+    return SC_OK;
+  };
   if (use_tail && per_layer && events == nullptr) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
@@ -609,9 +663,9 @@ static int stack_forward_impl(const sc_stack_args* a, void* workspace, size_t ws
       cap = cudaStreamCaptureStatusNone;
     }
     const int bound = per_layer_bound(a);
-    if (cap == cudaStreamCaptureStatusActive && bound >= 0) {
+    if (cap == cudaStreamCaptureStatusActive && bound >= 0 && a->pad_mask == nullptr) {
       direct = bound;
-      if (bound == a->n_layers && a->pad_mask == nullptr && !host_io) {
+      if (bound == a->n_layers && !host_io) {
         // no sequence gets short: the cluster kernel has nothing to do
         use_tail = false;
         tail_from = p.tail_from = pp.tail_from = nullptr;
@@ -620,20 +674,17 @@ static int stack_forward_impl(const sc_stack_args* a, void* workspace, size_t ws
     } else if (cap == cudaStreamCaptureStatusActive) {
       side = capture_side_stream();
     }
-    if (side != nullptr) {
-      cudaGraph_t g = nullptr;
-      cudaStreamCaptureStatus cs;
-      if ((e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &g)) != cudaSuccess)
-        return fail_cuda("stream capture info", e);
-      if ((e = cudaGraphConditionalHandleCreate(&cond, g, 0, cudaGraphCondAssignDefault)) !=
-          cudaSuccess)
-        return fail_cuda("conditional handle", e);
+    if (side != nullptr && bound >= 0) {
+      direct = bound;
+      group = a->keep_rule == SC_KEEP_TOP_RATIO ? kGroupLayers : bound;
+    } else if (side != nullptr) {
       dev_loop = true;
     }
+    if (side != nullptr && (rc = new_condition(&cond)) != SC_OK) return rc;
   }
   int* loop_layer = reinterpret_cast<int*>(ws + lay.loop_layer);
-  if (dev_loop) {
-    pp.dev_layer = loop_layer;
+  if (dev_loop) pp.dev_layer = loop_layer;
+  if (side != nullptr) {
     pp.cond = cond;
     pp.has_cond = 1;
   }
@@ -713,47 +764,22 @@ static int stack_forward_impl(const sc_stack_args* a, void* workspace, size_t ws
       if (le0 == cudaSuccess) le0 = launch_advance(ad, st);
       if (le0 != cudaSuccess) return fail_cuda("launch layer 0", le0);
     }
-    cudaGraph_t g = nullptr;
-    const cudaGraphNode_t* deps = nullptr;
-    size_t ndeps = 0;
-    cudaStreamCaptureStatus cs;
-    if ((e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, &deps, nullptr, &ndeps)) != cudaSuccess)
-      return fail_cuda("stream capture info", e);
-    cudaGraphNodeParams cp = {};
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = cond;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    cudaGraphNode_t node;
-    if ((e = cudaGraphAddNode(&node, g, deps, nullptr, ndeps, &cp)) != cudaSuccess)
-      return fail_cuda("add WHILE node", e);
-    if ((e = cudaStreamBeginCaptureToGraph(side, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
-                                           cudaStreamCaptureModeRelaxed)) != cudaSuccess)
-      return fail_cuda("capture layer loop body", e);
     // kLoopLayers layers a turn (those past the last, or that no sequence needs,
     // return at once)
-    cudaError_t le = cudaSuccess;
-    for (int k = 0; k < kLoopLayers && le == cudaSuccess; ++k) {
-      le = launch_rows(maps, pd, side);
-      if (le == cudaSuccess) le = launch_cols(maps, pd, side);
-      if (le == cudaSuccess) le = launch_gather(gd, side);
-      if (le == cudaSuccess) le = launch_advance(ad, side);
-    }
-    cudaGraph_t body = nullptr;
-    e = cudaStreamEndCapture(side, &body);
-    if (le != cudaSuccess) return fail_cuda("launch layer loop body", le);
-    if (e != cudaSuccess) return fail_cuda("end layer loop body capture", e);
-    if ((e = cudaStreamUpdateCaptureDependencies(st, &node, nullptr, 1,
-                                                 cudaStreamSetCaptureDependencies)) != cudaSuccess)
-      return fail_cuda("capture dependencies", e);
+    rc = add_conditional(cudaGraphCondTypeWhile, cond, [&]() -> int {
+      cudaError_t le = cudaSuccess;
+      for (int k = 0; k < kLoopLayers && le == cudaSuccess; ++k) {
+        le = launch_rows(maps, pd, side);
+        if (le == cudaSuccess) le = launch_cols(maps, pd, side);
+        if (le == cudaSuccess) le = launch_gather(gd, side);
+        if (le == cudaSuccess) le = launch_advance(ad, side);
+      }
+      return le == cudaSuccess ? SC_OK : fail_cuda("launch layer loop body", le);
+    });
+    if (rc != SC_OK) return rc;
   }
-  for (int l = 0; l < a->n_layers; ++l) {
-    if (dev_loop || l >= direct) break;
-    if (!per_layer) {
-      if (!mark(2 + 3 * l) || !mark(3 + 3 * l) || !mark(4 + 3 * l))
-        return fail(SC_ERR_CUDA, "event record", "");
-      continue;
-    }
+  // layer l and the gather of the next layer's rows, on s
+  auto launch_layer = [&](int l, cudaStream_t s) -> int {
     fill_workspace(&p, ws, lay, l & 1);
     p.gathered = nullptr;   // only layer 0 of a host-buffer call counts its rows in
     p.layer = l;
@@ -774,14 +800,14 @@ static int stack_forward_impl(const sc_stack_args* a, void* workspace, size_t ws
       gp.pos = p.pos;
       gp.ident = p.ident;
       gp.gathered = gathered;
-      if ((e = launch_gather(gp, st)) != cudaSuccess) return fail_cuda("launch gather kernel", e);
+      if ((e = launch_gather(gp, s)) != cudaSuccess) return fail_cuda("launch gather kernel", e);
       gp.gathered = nullptr;
       p.gathered = gathered;
       p.gather_target = gather_target;
     }
-    if ((e = launch_rows(maps, p, st)) != cudaSuccess) return fail_cuda("launch rows kernel", e);
+    if ((e = launch_rows(maps, p, s)) != cudaSuccess) return fail_cuda("launch rows kernel", e);
     if (!mark(2 + 3 * l)) return fail(SC_ERR_CUDA, "event record", "");
-    if ((e = launch_cols(maps, p, st)) != cudaSuccess) return fail_cuda("launch cols kernel", e);
+    if ((e = launch_cols(maps, p, s)) != cudaSuccess) return fail_cuda("launch cols kernel", e);
     if (!mark(3 + 3 * l)) return fail(SC_ERR_CUDA, "event record", "");
     if (l + 1 < direct) {
       gp.src_base = static_cast<long long>(l + 1) * BLt;
@@ -789,9 +815,37 @@ static int stack_forward_impl(const sc_stack_args* a, void* workspace, size_t ws
       gp.len = p.len_out;
       gp.pos = p.pos_out;
       gp.ident = p.ident_out;
-      if ((e = launch_gather(gp, st)) != cudaSuccess) return fail_cuda("launch gather kernel", e);
+      if ((e = launch_gather(gp, s)) != cudaSuccess) return fail_cuda("launch gather kernel", e);
     }
     if (!mark(4 + 3 * l)) return fail(SC_ERR_CUDA, "event record", "");
+    return SC_OK;
+  };
+  for (int l = 0; !dev_loop && l < direct;) {
+    if (!per_layer) {
+      if (!mark(2 + 3 * l) || !mark(3 + 3 * l) || !mark(4 + 3 * l))
+        return fail(SC_ERR_CUDA, "event record", "");
+      ++l;
+      continue;
+    }
+    // layers l .. upto - 1: in a node of their own where they are conditional
+    const int upto = group == 0 ? l + 1 : std::min(direct, l + group);
+    auto launch_group = [&](cudaStream_t s) -> int {
+      for (; l < upto; ++l)
+        if ((rc = launch_layer(l, s)) != SC_OK) return rc;
+      if (group == 0 || upto >= direct) return SC_OK;
+      AdvanceParams ad{};
+      ad.B = a->B;
+      ad.n_layers = a->n_layers;
+      ad.layer = upto;
+      ad.tail_from = tail_from;
+      if ((rc = new_condition(&cond)) != SC_OK) return rc;   // of the next group
+      ad.cond = cond;
+      e = launch_advance(ad, s);
+      return e == cudaSuccess ? SC_OK : fail_cuda("launch advance kernel", e);
+    };
+    if (group == 0) rc = launch_group(st);
+    else rc = add_conditional(cudaGraphCondTypeIf, cond, [&]() { return launch_group(side); });
+    if (rc != SC_OK) return rc;
   }
   if (use_tail) {
     TailParams tp{};

@@ -180,12 +180,15 @@ struct GatherParams {
 };
 
 // One step of the device-driven layer loop: layer += 1, and the loop goes on
-// while some sequence still runs through the per-layer kernels.
+// while some sequence still runs through the per-layer kernels.  Without a loop
+// (dev_layer == nullptr) the layer is given, and the condition is that of the
+// graph node that holds the layers from there on.
 struct AdvanceParams {
   int B, n_layers;
   int* dev_layer;
+  int layer;
   const int32_t* tail_from;
-  unsigned long long cond;     // cudaGraphConditionalHandle of the WHILE node
+  unsigned long long cond;     // cudaGraphConditionalHandle of the WHILE (IF) node
 };
 
 struct PrepParams {

@@ -1510,14 +1510,14 @@ __global__ void __launch_bounds__(256) sc_advance_kernel(const AdvanceParams a) 
   pdl_launch_dependents();
   pdl_wait();
   __shared__ int s_layer;
-  if (threadIdx.x == 0) s_layer = __ldcg(a.dev_layer) + 1;
+  if (threadIdx.x == 0) s_layer = a.dev_layer != nullptr ? __ldcg(a.dev_layer) + 1 : a.layer;
   __syncthreads();
   const int l = s_layer;
   int big = 0;
   for (int b = threadIdx.x; b < a.B; b += blockDim.x) big |= __ldcg(a.tail_from + b) > l;
   big = __syncthreads_or(big);
   if (threadIdx.x == 0) {
-    *a.dev_layer = l;
+    if (a.dev_layer != nullptr) *a.dev_layer = l;
     cudaGraphSetConditional(a.cond, (big && l < a.n_layers) ? 1u : 0u);
   }
 }

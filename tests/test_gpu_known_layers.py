@@ -69,3 +69,40 @@ def test_graph_equals_plain_launches(nl, L, lens, rule, alphas, host):
             # every layer stays with the per-layer kernels in both (nothing gets short)
             assert int(a["len"][:-1].min()) == L
         assert torch.equal(x, y), k
+
+
+def _graph_nodes(graph):
+    import ctypes
+    n = ctypes.c_size_t(0)
+    rt = ctypes.CDLL("libcudart.so.13")   # the one that the library has loaded
+    assert rt.cudaGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), None, ctypes.byref(n)) == 0
+    return n.value
+
+
+@pytest.mark.parametrize("rule,alpha,groups", [(RELATIVE, 0.0, 1), (TOP_RATIO, 0.95, 2)])
+def test_padded_stack_bounds_are_conditional(rule, alpha, groups):
+    """With padding the bound comes from L and the true lengths may be short: the
+    layers sit in conditional nodes beside the padding removal and the cluster
+    kernel, so that a batch of short sequences launches none of them."""
+    import paper_2310_07109_gb300 as sc
+    nl, B, L, H = 12, 2, 2048, 2
+    Q, K, V = (torch.zeros((nl, B, L, H, 64), device="cuda", dtype=torch.bfloat16)
+               for _ in range(3))
+    mask = torch.zeros((B, L), dtype=torch.uint8, device="cuda")
+    mask[:, :300] = 1
+    ws = sc.new_workspace(B, L, H)
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        out = sc.stack_forward(Q, K, V, mask, [0], 64, [alpha] * nl, workspace=ws, keep_rule=rule)
+    assert _graph_nodes(graph) == 3 + groups   # with the counters' reset
+    for n in (300, 1500, 2048):    # the same graph, other lengths
+        mask.zero_()
+        mask[:, :n] = 1
+        graph.replay()
+        torch.cuda.synchronize()
+        assert sc.workspace_status(ws) == 0
+        want = [n]
+        for _ in range(nl):
+            r = torch.tensor(alpha, dtype=torch.float32).double().item()
+            want.append(want[-1] if rule == RELATIVE else -int(-r * want[-1] // 1))
+        assert out["len"][:, 0].tolist() == want
