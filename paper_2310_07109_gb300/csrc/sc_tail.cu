@@ -586,7 +586,6 @@ __global__ void __launch_bounds__(kTailThreads, 1)
         sm.nlse[i] = me.valid ? -(ref + lg2(lsum)) : -INFINITY;
         if (!(ok = tail_wait(&sm.bar_odone[X], (n_odone++) & 1, abort_flag))) break;
         tc_fence_after();
-        if (o_held) store_o();              // the warpgroup's first query tile of two
         const float inv = me.valid ? 1.f / osum : 0.f;
 #pragma unroll
         for (int c = 0; c < 64; c += 32) {
@@ -597,12 +596,15 @@ __global__ void __launch_bounds__(kTailThreads, 1)
           for (int k = 0; k < 32; k += 2)
             opk[(c + k) >> 1] = pack_bf16x2(o[k] * inv, o[k + 1] * inv);
         }
-        // O is in registers: the columns may take S^T; O is stored while the
-        // cluster's column sums are awaited
+        // O is in registers: the columns may take the next product.  It is stored
+        // while that runs (the first query tile of two; ahead of the second tile's O
+        // it took 8 sequences of 384 tokens, 12 layers, all pairs allowed, 296 us
+        // instead of 290), or while the cluster's column sums are awaited
         release();
-        o_held = true;
         o_row = i - (r & 31);
         o_rows = __ballot_sync(0xffffffffu, me.valid);
+        o_held = qt + 2 >= nq;
+        if (!o_held) store_o();
       }
       // rows past the last query tile take no part in the column sums
       for (int i = kTile * nq + (tid & 255); i < kTailMax; i += 256) sm.nlse[i] = -INFINITY;
