@@ -40,6 +40,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -336,6 +337,46 @@ class ClockSampler:
 # ---------------------------------------------------------------------------
 # CPU oracle (the reference arm and the cpu_baseline)
 # ---------------------------------------------------------------------------
+def graph_launch_count(wl, lens, tail_max: int, padded: bool) -> int:
+    """Kernels that one stack call launches as a graph, from the lengths it gave.
+
+    The removal of padding comes first and the cluster kernel last; between them,
+    while some sequence has more than ``tail_max`` tokens, rows + scores + gather
+    per layer.  Where the rule bounds the layers from L (the top-ratio rule; no
+    threshold above 0 but in the last layer) just these are recorded, without a
+    gather after the last, and without the cluster kernel where that is every layer;
+    with padding they sit in conditional groups (six layers under the top-ratio
+    rule, else all), whose conditions an advance kernel at the end of the group
+    before sets.  Otherwise layer 0, then a loop of two layers a turn, each with
+    an advance kernel."""
+    nl, alphas = wl.n_layers, np.float32(wl.alphas())
+    if wl.L <= tail_max:
+        return 2
+    longer = [bool((np.asarray(lens[l]) > tail_max).any()) for l in range(nl)]
+    bound = None
+    if wl.keep_rule == 2:
+        bound, n = 0, wl.L
+        while bound < nl and n > tail_max:
+            n = min(n, max(1, math.ceil(float(alphas[bound]) * n)))
+            bound += 1
+    elif (alphas[:-1] <= 0).all():
+        bound = nl
+    if bound is None:
+        return 1 + padded + 4 * (1 + 2 * (sum(longer[1:]) + 1 >> 1)) + 1
+    if not padded:
+        return 1 + 3 * bound - 1 + (bound < nl)
+    group = 6 if wl.keep_rule == 2 else bound
+    count = 2
+    for first in range(0, bound, group):
+        if not longer[first]:
+            break
+        last = min(bound, first + group)
+        # the gather of layer 0's rows, and per group an advance kernel or, at the
+        # end, one gather less
+        count += (first == 0) + 3 * (last - first) + (1 if last < bound else -1)
+    return count
+
+
 def oracle_sample(wl, inp, b, n_layers, threads):
     """Run the oracle stack on sequence b for the first n_layers layers; returns
     (seconds, kept tokens processed, threads used)."""
@@ -533,25 +574,11 @@ def run_native(args, wl):
     kept_per_step = int(lens[:wl.n_layers].sum())
     value = whole_job_rate(world, kept_per_step, ms_per_step)
 
-    # ---- kernels launched per timed step.  A captured step, and an eager call
-    # (which the library records into a graph of its own): prep, [padding
-    # gather], then rows + scores + gather for every layer that the arguments
-    # let need them, or, where they do not tell, rows + scores + gather + advance
-    # for layer 0 and for pairs of later layers while some sequence has more than
-    # TAIL_MAX_LEN tokens, then the cluster kernel.  With plain launches: the
-    # library's plan.
+    # ---- kernels launched per timed step (a captured step and an eager call are
+    # graphs; with plain launches: the library's plan)
     eager_launches = sc.stack_launch_count(wl.n_layers, wl.B, wl.L, wl.H, wl.w, gpos,
                                            inp["pad_mask"] is not None)
-    looped = sum(1 for l in range(wl.n_layers) if (lens[l] > sc.TAIL_MAX_LEN).any())
-    pad = 1 if inp["pad_mask"] is not None else 0
-    if wl.L <= sc.TAIL_MAX_LEN:
-        graph_launches = 2
-    elif wl.keep_rule == sc.SC_KEEP_TOP_RATIO:
-        graph_launches = 1 + pad + 3 * looped - 1 + 1   # no gather after the last
-    elif all(a <= 0 for a in wl.alphas()[:-1]):
-        graph_launches = 1 + pad + 3 * wl.n_layers - 1 + pad
-    else:
-        graph_launches = 1 + pad + 4 * (1 + 2 * ((looped - 1 + 1) // 2)) + 1
+    graph_launches = graph_launch_count(wl, lens, sc.TAIL_MAX_LEN, inp["pad_mask"] is not None)
     launches_per_step = (eager_launches if graph is None and args.plain_launches
                          else graph_launches)
 
