@@ -18,6 +18,9 @@
  * - Arguments are validated on the host before anything is launched; a bad
  *   argument returns an SC_ERR_* code with nothing enqueued.  CUDA launch
  *   errors return SC_ERR_CUDA.  No C++ exception crosses this interface.
+ * - A NaN or infinity in the row of a current token may reach rows of O that do
+ *   not attend to it (the products run over whole tiles, with P = 0 outside a
+ *   row's allowed keys).
  * - Every wait inside a kernel is bounded (about 2 s).  A wait that expires
  *   makes the kernel record SC_ERR_TIMEOUT in the workspace status word and
  *   return; sc_workspace_status() reports (and clears) it.
@@ -80,7 +83,8 @@ typedef enum {
  * One layer on tokens already in current (compacted) order.
  *
  * Q, K, V    bf16 [B][L][H][64]; row c of sequence b holds current token c.
- *            Rows at or beyond len[b] are never read.
+ *            Rows at or beyond len[b] reach no result, whatever they hold (they
+ *            may be NaN).
  * len        int32 [B]: current length n_b (0 <= n_b <= L).
  * pos        int32 [B][L]: original position of each current token, strictly
  *            increasing within [0, n_b).  Decides which tokens are global and
@@ -245,7 +249,9 @@ int sc_layer_forward(const sc_layer_args* args, void* workspace, size_t workspac
  * layers a turn), so the layers that every sequence runs in the cluster kernel
  * launch nothing; where the arguments bound the layers that can need the
  * per-layer kernels (the top-ratio rule; thresholds <= 0 in every layer but the
- * last), just those are launched, without a loop.
+ * last), just those are launched, without a loop, and with a pad_mask (the bound
+ * is then that of L, not of the true lengths) in groups of layers that run only
+ * while some sequence is longer than SC_TAIL_MAX_LEN.
  * An eager call (stream not capturing) that has both kinds of kernels in its
  * plan runs the same way: the library records the call into a graph of its
  * own, keeps the instantiated graph (up to 16 per process, least recently
@@ -280,12 +286,13 @@ int sc_stack_forward_profiled(const sc_stack_args* args, void* workspace, size_t
  * current device) when it launches them directly (SC_STACK_PLAIN_LAUNCHES, or
  * a plan with one kind of kernel), in *count.  A call that runs as a graph
  * launches prep, [padding-removal gather], then rows, scores and gather for each
- * layer whose need the arguments bound, or rows, scores, gather and a
- * loop-advance kernel for layer 0 and for pairs of later layers while some
- * sequence still runs per layer, then the cluster kernel.  Only the sizes, n_layers,
- * flags, pad_mask (NULL or not) and the global list are read; no pointer is
- * dereferenced and nothing is launched.  Errors: see sc_status (SC_ERR_CUDA
- * without a usable device). */
+ * layer whose need the arguments bound (and an advance kernel between groups of
+ * them), or rows, scores, gather and a loop-advance kernel for layer 0 and for
+ * pairs of later layers while some sequence still runs per layer, then the cluster
+ * kernel (unless every layer is known to stay with the per-layer kernels).  Only
+ * the sizes, n_layers, flags, pad_mask (NULL or not) and the global list are read;
+ * no pointer is dereferenced and nothing is launched.  Errors: see sc_status
+ * (SC_ERR_CUDA without a usable device). */
 int sc_stack_launch_count(const sc_stack_args* args, int* count);
 
 /*
@@ -376,7 +383,7 @@ int sc_workspace_status(void* workspace, size_t workspace_bytes, void* stream);
  * gathered in its epilogue), layer norm, the two feed-forward GEMMs, layer norm.
  *
  * X          bf16 [B][L][D] hidden states in current order (row c of sequence b
- *            is current token c; rows at or beyond len[b] are never read).
+ *            is current token c; rows at or beyond len[b] reach no result).
  * len, pos, w, global_pos, n_global, keep_rule, alpha, theta: as sc_layer_args.
  * W_qkv bf16 [3D][D], b_qkv fp32 [3D]; W_o bf16 [D][D], b_o [D];
  * ln1_gamma, ln1_beta fp32 [D]; W_1 bf16 [4D][D], b_1 [4D]; W_2 bf16 [D][4D],

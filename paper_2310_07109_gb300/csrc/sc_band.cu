@@ -31,10 +31,9 @@
 // block share the row's running reference through shared memory), 8-11
 // helpers (the previous tile's epilogue), 12 loads Q, the global rows and the
 // K ring, 13 issues the S and P V products, 14 loads the V ring, 15 holds the
-// tensor memory and issues the column-sum products.  Its outputs are those of
-// the paired rows kernel (O, the band rows' column sums per query tile, the
-// global keys' far-row sums, the global queries' (max, sum) pieces), so the
-// cols kernel is the same for both.
+// tensor memory and issues the column-sum products.  The cols kernel behind it
+// takes the band rows' column sums per query tile, the global keys' far-row sums
+// and the global queries' (max, sum) pieces.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <cstdint>

@@ -30,12 +30,12 @@ constexpr int kTailMax = SC_TAIL_MAX_LEN;
 constexpr int kTailMaxLayers = 64;
 constexpr int kTailMaxHeads = 16;   // largest (non-portable) cluster
 
-// log2(e) / sqrt(64): logits are kept in base-2 units, x = (q.k) * kLogitScale2.
 // keep rules (the SC_KEEP_* values of the C interface)
 constexpr int kKeepRelative = SC_KEEP_RELATIVE;
 constexpr int kKeepAbsolute = SC_KEEP_ABSOLUTE;
 constexpr int kKeepTopRatio = SC_KEEP_TOP_RATIO;
 
+// log2(e) / sqrt(64): logits are kept in base-2 units, x = (q.k) * kLogitScale2.
 constexpr float kLogitScale2 = 0.125f * 1.4426950408889634f;
 
 // TMA descriptors of Q, K, V (index 0, 1, 2) for both row sources: [0] the
@@ -130,7 +130,7 @@ struct LayerParams {
   float alphas[kTailMaxLayers];
 };
 
-// The per-layer fields of one launch, resolved (see layer_view in sc_kernels.cu).
+// The per-layer fields of one launch, resolved (see layer_view in sc_layer_common.cuh).
 struct LayerView {
   int layer;
   long long src_base;
@@ -286,7 +286,6 @@ struct GemmParams {
   int* status;
 };
 
-// Layer norm over D features of the rows (b, r), r < rows[b]: fp32 in, bf16 out.
 // Rows of a bf16 [B L][D] matrix gathered into consecutive rows:
 // dst[b L + r] = src[b L + idx[b L + r]] for r < rows[b].
 struct RowGatherParams {
@@ -297,6 +296,7 @@ struct RowGatherParams {
   uint16_t* dst;
 };
 
+// Layer norm over D features of the rows (b, r), r < rows[b]: fp32 in, bf16 out.
 struct LayerNormParams {
   int B, L, D;
   const int32_t* rows;

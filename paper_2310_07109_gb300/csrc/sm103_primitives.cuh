@@ -105,19 +105,6 @@ __device__ __forceinline__ bool mbar_try_wait_poll(uint64_t* bar, uint32_t parit
   return ok != 0;
 }
 
-// Non-blocking: whether the phase with the given parity has completed.
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
 // Wait for the phase with the given parity to complete, for at most
 // `limit_ns` of wall time.  Gives up early when another role of the CTA has
 // already raised `*abort` (a shared-memory flag).  On expiry raises `*abort`
@@ -235,10 +222,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
-}
-
-__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -450,14 +433,6 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
 // ---------------------------------------------------------------------------
 // thread-block clusters and L2 prefetch
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-
-// Every thread of every CTA of the cluster arrives (release) and waits
-// (acquire); called by whole, converged warps.
 // Split cluster barrier: arrive without ordering (only "this CTA is running"),
 // and the matching wait.
 __device__ __forceinline__ void cluster_arrive_relaxed() {
@@ -467,6 +442,8 @@ __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 }
 
+// Every thread of every CTA of the cluster arrives (release) and waits
+// (acquire); called by whole, converged warps.
 __device__ __forceinline__ void cluster_sync() {
   asm volatile(
       "barrier.cluster.arrive.release.aligned;\n\t"
@@ -479,12 +456,6 @@ __device__ __forceinline__ uint32_t dsmem_addr(uint32_t saddr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
-}
-
-__device__ __forceinline__ float ld_dsmem_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
 }
 
 // A store into another CTA's shared memory that counts its 4 bytes on an mbarrier
@@ -535,18 +506,6 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // Hint: bring the 128-byte line holding `gptr` into L2.
 __device__ __forceinline__ void prefetch_l2_line(const void* gptr) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(gptr));
-}
-
-// Four fp32 atomic additions to 16-byte aligned global memory in one request.
-__device__ __forceinline__ void red_add_v4(float* gptr, float a, float b, float c, float d) {
-  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(gptr), "f"(a), "f"(b),
-               "f"(c), "f"(d)
-               : "memory");
-}
-
-// Bring `bytes` (a multiple of 16, 16-byte aligned) of global memory into L2.
-__device__ __forceinline__ void prefetch_l2(const void* gptr, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gptr), "r"(bytes) : "memory");
 }
 
 // ---------------------------------------------------------------------------
