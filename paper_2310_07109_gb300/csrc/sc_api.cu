@@ -601,8 +601,8 @@ static int stack_forward_impl(const sc_stack_args* a, void* workspace, size_t ws
   // Where the arguments bound the layers that can need those kernels, a captured
   // call records just these layers one after the other, without the loop, whose
   // every turn costs about 7 us beside its kernels (3 x 1000 tokens, nothing
-  // pruned, 12 layers: 371 us with the loop, 286 without; 4 x 777, top ratio:
-  // 428 and 381).
+  // pruned, 12 layers: 338 us with the loop, 264 without; 4 x 777, top ratio:
+  // 415 and 365).
   // With padding the bound holds for L and not for the true lengths, so there the
   // layers run only where some sequence is longer than kTailMax: all of them in
   // one IF node where nothing is pruned, in groups of kGroupLayers under the

@@ -180,10 +180,10 @@ __device__ __forceinline__ void gemm_plan(const GemmParams& p, GemmSmem& sm, int
   // round.  Widths divide N and the split blocks; with a gathered A, 256 (A is
   // fetched again for every column tile).  One width per lane.  A short batch
   // leaves most SMs idle and each busy one fetches at its own L2 rate, so there
-  // the narrowest tiles win: a layer of one sequence of 200 tokens takes 67.5 us
-  // with 64-column tiles and 77.2 with 128 as the narrowest.  Counting the rows
+  // the narrowest tiles win: a layer of one sequence of 200 tokens takes 60.9 us
+  // with 64-column tiles and 67.9 with 128 as the narrowest.  Counting the rows
   // that are there, not the L there may be, gives a layer of 8 x 1024 tokens with
-  // a third pruned 198 us instead of 212.
+  // a third pruned 172 us instead of 178.
   uint32_t key = 0xffffffffu;
   const int c = kGemmBN - 64 * lane;
   if (c > 0 && (p.a_idx == nullptr || c == kGemmBN)) {

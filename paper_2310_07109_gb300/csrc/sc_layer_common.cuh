@@ -110,7 +110,8 @@ __device__ __forceinline__ void load_tile(const TensorMaps& m, int t, const RowS
 // matrix products that follow (the caller is a whole warp, or one thread as lane 0
 // of 1, and the tile has landed).  P V multiplies whole 16-row blocks: rows past the
 // sequence's end have P = 0, but 0 x Inf and 0 x NaN are NaN, and what lies there is
-// the caller's padding, another sequence or an earlier use of the workspace.
+// the caller's padding, another sequence or an earlier use of the workspace.  It
+// costs 0.1 us a layer (3 x 1000 tokens, 12 layers: 261.6 us without, 262.5 with).
 __device__ __forceinline__ void zero_rows(uint8_t* tile, int from, int to, int lane, int lanes) {
 #pragma unroll 1
   for (int k = 8 * from + lane; k < 8 * to; k += lanes)

@@ -61,9 +61,12 @@ static_assert(kTailDyn > 233472 / 2, "the tail kernel must occupy an SM alone");
 // Windows of kWideWindow and more have an instance whose layers of more than
 // kWideFrom tokens take 64 columns at a time, unrolled, without a test for empty
 // chunks (there are next to none): 12 layers, 8 sequences of 384 tokens, nothing
-// pruned, all pairs allowed 297 us instead of 321.  Smaller layers, and narrow
-// windows, lose by the longer code (24 x 128, w = 64: 218 instead of 210, even
-// where the wide loops are in the kernel but not taken): hence the instance.
+// pruned, all pairs allowed 290 us instead of 314; 320 tokens at w = 200 279
+// instead of 294.  Smaller layers, and narrow windows, lose by the longer code
+// (24 x 128, w = 64: 267.5 instead of 259.5 us, 16 x 333 pruned 621 instead of 558,
+// even where the wide loops are in the kernel but not taken): hence the instance.
+// From w = 128 on it would be slower (8 x 384 at w = 128 328 instead of 323; at
+// w = 160 323 instead of 325).
 constexpr int kWideWindow = 192, kWideFrom = 192;
 
 struct TailSmem {
@@ -394,9 +397,10 @@ __global__ void __launch_bounds__(kTailThreads, 1)
       // exactly); half 1 raises it to its own maximum when that lies more than 8
       // above, O and the sums being rescaled.  The first pass writes the scores
       // back masked, and the second neither masks nor looks at windows again: a
-      // 12-layer stack of 16 x 333 tokens takes 275 us so, 292 with the masks
-      // applied twice, and 273 with a reference from the first chunk alone, which
-      // made O's error against 64 bits 2 to 4 % larger.
+      // 12-layer stack of 16 x <= 333 tokens takes 288 us so and 303 with the masks
+      // applied twice, 1 x 96 65.9 and 67.8 (both builds in turn on one GPU).  A
+      // reference from the first chunk alone was half a percent faster and made O's
+      // error against 64 bits 2 to 4 % larger.
       // lsum: the sum of the exponentials (fp32: the row's LSE, which the column
       // sums use); osum: the sum of the same values rounded to the bf16 that P V
       // multiplies (the normaliser of O, so that O is a weighted mean of V rows
