@@ -70,7 +70,7 @@ struct LayerParams {
   const float* theta;    // [B] absolute thresholds or nullptr (threshold rules)
   int keep_rule;         // kKeepRelative, kKeepAbsolute or kKeepTopRatio
   // workspace
-  float* acc;            // [B][H][L] per-head column sums: band rows + global rows
+  float* acc;            // with band: [B][H][L] per-head column sums: band rows + global rows
   float* colpart;        // [B][H][band_slots][L] band-row column sums per query tile
                          //   (slot = query tile mod band_slots); with band:
                          //   [B][H][L][kMaxBandTiles]
@@ -89,11 +89,11 @@ struct LayerParams {
   float* gog;            // [B][H][T][kMaxGlobal][64] fp32 parts of the global rows' outputs, one
                          //   per key tile, relative to the same maximum
   uint8_t* keep;         // [B][L]
-  uint32_t* cnt_tile;    // [B][T]
+  uint32_t* cnt_tile;    // with band: [B][T]
   uint32_t* cnt_seq;     // [B]
   uint32_t* rows_done;   // [B][H]: rows CTAs of a sequence whose results are visible (the
                          //   first entry of each sequence; with band: of each (sequence, head))
-  uint32_t* cols_done;   // [B][H]: cols CTAs of (sequence, head) whose global-row parts are stored
+  uint32_t* cols_done;   // with band: [B][H]: cols CTAs whose global-row parts are stored
   // nonzero: the gather kernel before this launch is still copying later
   // sequences' rows when it starts: sequence b's rows are complete once
   // gathered[b] reaches gather_target (the attention kernels wait for it

@@ -543,7 +543,8 @@ __global__ void __launch_bounds__(kRowsThreads, 2)
     // reference, every row of the warp that lies below its own maximum takes that
     // as its reference, and the row sums and O are rescaled: O after the item's
     // exponentials, when the P V before it is long complete.  So P stays below
-    // 2^kRefSlack.
+    // 2^kRefSlack.  (The reference of a row, and with it the last bits of its O,
+    // thus depends on the 31 rows of its warp too.)
     // Only the element the reference comes from is exact in bf16, so a reference
     // nearer to the maximum makes O's error smaller; at 6 the error against 64
     // bits is that of whole-tile items raised past 2^8.  12 layers of 8 x 1024

@@ -63,10 +63,10 @@ static_assert(kTailDyn > 233472 / 2, "the tail kernel must occupy an SM alone");
 // chunks (there are next to none): 12 layers, 8 sequences of 384 tokens, nothing
 // pruned, all pairs allowed 290 us instead of 314; 320 tokens at w = 200 279
 // instead of 294.  Smaller layers, and narrow windows, lose by the longer code
-// (24 x 128, w = 64: 267.5 instead of 259.5 us, 16 x 333 pruned 621 instead of 558,
-// even where the wide loops are in the kernel but not taken): hence the instance.
-// From w = 128 on it would be slower (8 x 384 at w = 128 328 instead of 323; at
-// w = 160 323 instead of 325).
+// (24 x 128, w = 64: 267.5 instead of 259.5 us, 16 x 333 with flat scores 621
+// instead of 558, even where the wide loops are in the kernel but not taken): hence
+// the instance.  A lower limit gains nothing (8 x 384 at w = 128 328 instead of 323
+// us, at w = 160 323 instead of 325).
 constexpr int kWideWindow = 192, kWideFrom = 192;
 
 struct TailSmem {

@@ -40,7 +40,9 @@ def test_layer_edges(L, lens, w, gl, scale, H):
     Q, K, V = (bits_to_torch(case[k], "cuda") for k in ("Q", "K", "V"))
     length, pos = (torch.from_numpy(case[k]).cuda() for k in ("len", "pos"))
     ws = sc.new_workspace(B, L, H)
-    ws.fill_(255)      # whatever the workspace holds, no result may depend on it
+    # whatever the scratch of the partial results holds, no result may depend on it
+    # (a layer reads the caller's rows: test_gpu_stale_rows.py covers compacted ones)
+    ws.fill_(255)
     ws[:256] = 0       # (but for the status word)
     O, s, po, lo = sc.layer_forward(Q, K, V, length, pos, w, case["global_pos"], 0.8, workspace=ws)
     assert sc.workspace_status(ws) == 0
