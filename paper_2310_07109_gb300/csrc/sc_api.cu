@@ -506,11 +506,6 @@ struct HostResults {
   int32_t* len;
 };
 
-// host_io: Q, K, V (and pad_mask) are device-mapped addresses of host memory,
-// which only the gather and cluster kernels read (plain loads): the tensor
-// maps of the "source" slot are pointed at the compacted copies and never
-// selected, and every layer's rows are gathered; hres (host_io only): where
-// the cluster kernel puts its results.
 // The argument checks of a stack call (nothing is enqueued).
 static int stack_check(const sc_stack_args* a, void* workspace, size_t ws_bytes) {
   if (!a) return SC_ERR_INVALID_ARG;
@@ -533,6 +528,11 @@ static int stack_check(const sc_stack_args* a, void* workspace, size_t ws_bytes)
   return ensure_configured();
 }
 
+// host_io: Q, K, V (and pad_mask) are device-mapped addresses of host memory,
+// which only the gather and cluster kernels read (plain loads): the tensor
+// maps of the "source" slot are pointed at the compacted copies and never
+// selected, and every layer's rows are gathered; hres (host_io only): where
+// the cluster kernel puts its results.
 static int stack_forward_impl(const sc_stack_args* a, void* workspace, size_t ws_bytes,
                               void* stream, void** events, int n_events, bool host_io = false,
                               const HostResults* hres = nullptr) {
@@ -628,7 +628,7 @@ static int stack_forward_impl(const sc_stack_args* a, void* workspace, size_t ws
   // a WHILE or IF node after the work captured on st so far, whose body is what
   // `body` launches on the side stream
   auto add_conditional = [&](cudaGraphConditionalNodeType type, cudaGraphConditionalHandle h,
-                             const std::function<int()>& body) -> int {
+                             auto&& body) -> int {
     cudaGraph_t g = nullptr;
     const cudaGraphNode_t* deps = nullptr;
     size_t ndeps = 0;
